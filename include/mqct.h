@@ -420,8 +420,9 @@ mqct_status mqct_cross_sections(mqct_system sys, const double *final_pop, const 
  * spline through (U_k, sigma_sym[k][a][b]) (negative values taken as zero); below U_1 it falls
  * linearly to zero at the threshold u0 = |E_b - E_a|/2 (or the spline is cut at u0 when
  * u0 >= U_1); above U_K it continues as sigma_sym[K-1] (U/U_K)^p, p the log-log slope of the
- * last two points clipped to [-1, 0].  The finite pieces are integrated by Gauss-Legendre
- * panels no wider than 4 kT (relative error below ~1e-13), the tail in closed form.
+ * last two points clipped to [-1, 0].  The integral is taken in closed form where the spline is shown
+ * non-negative (relative error below ~1e-13), else its finite pieces by Gauss-Legendre panels no wider than
+ * 4 kT and the tail in closed form.
  *
  * sigma [K][L][L] (host or device); sigma_sym [K][L][L] output, or NULL to skip it;
  * rate [n_temps][L][L] output, rate[t][a][b] = k_{a->b}(T_t) in bohr^3 per atomic unit of time

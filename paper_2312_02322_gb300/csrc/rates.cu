@@ -14,13 +14,23 @@
 //   R5  above U_K the power law sigma~_K (U/U_K)^p, p the log-log slope of the last two points
 //       clipped to [-1, 0], integrated in closed form with the upper incomplete gamma function.
 //
-// One thread per (unordered pair of levels, temperature).  The spline's second derivatives are
-// a fixed linear map of the knot values (set up on the host from the energy grid), the finite
-// pieces are integrated by 16-point Gauss-Legendre panels no wider than 4 kT (the exponential at the
-// nodes as a panel factor times node factors shared by the panels of a piece), and the integrand
-// carries exp(-(U - u0)/kT) so that neither exponential factor of R2 overflows.  The walk stops at
-// the first panel whose remainder bound (4 max|y| kT (U + kT) exp(-(U - u0)/kT) at its lower edge U)
-// is below 1e-17 of the integral so far; the tail is then dropped too.
+// One thread per unordered pair of levels and chunk of temperatures.  The spline's second derivatives
+// are a fixed linear map of the knot values (set up on the host from the energy grid).  Two forms of
+// the integral:
+//   closed form  when no piece of the spline at or above u0 can be negative (its Bernstein coefficients
+//       are >= 0, so the cubic is): the integral over every whole piece is linear in the knot values with
+//       weights that depend on the temperature alone (host tables, rate_tables); the piece that u0
+//       cuts (or the ramp) is a quartic times exp(-(U - u0)/kT), i.e. five lower incomplete gamma functions
+//       of integer order; the tail's Gamma(2 + p, U_K/kT) is a Chebyshev series in p per temperature.
+//       About 170 FP64 instructions per pair and temperature instead of about 4400: the kernel is bound
+//       by the FP64 pipe, so the instruction count is its time.
+//   quadrature  for every other pair (a value below zero is taken as zero, R3), a u0 at or above U_K, and
+//       temperatures or energies outside [1e-12, 1e6] hartree: 16-point Gauss-Legendre panels no
+//       wider than 4 kT (the exponential at the nodes as a panel factor times node factors shared by the
+//       panels of a piece); the walk stops at the first panel whose remainder bound
+//       (4 max|y| kT (U + kT) exp(-(U - u0)/kT) at its lower edge U) is below 1e-17 of the integral so
+//       far; the tail is then dropped too.
+// The integrand carries exp(-(U - u0)/kT) so that neither exponential factor of R2 overflows.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,16 +47,28 @@ namespace {
 constexpr int kRateMaxK = MQCT_RATE_MAX_ENERGIES;
 constexpr int kRateMaxT = MQCT_RATE_MAX_TEMPS;
 constexpr int kGl = 16;
+constexpr int kRateThreads = 128;          // a block's tile of pairs: 16 levels a x 8 levels b
+constexpr int kRateTa = 16, kRateTb = 8;
+constexpr int kRateCheb = 16;              // Chebyshev coefficients of the tail per temperature
 
 struct RateArgs {
     double u[kRateMaxK];
     double Q[kRateMaxK][kRateMaxK];  // second derivatives of the natural spline: M = Q y
     double gx[kGl], gw[kGl];         // Gauss-Legendre nodes and weights on [-1, 1]
     double kT[kRateMaxT];
-    double pref;                     // (8 / (pi mu))^(1/2)
+    double ikT[kRateMaxT];           // 1 / kT
+    double pref[kRateMaxT];          // (8 / (pi mu))^(1/2) kT^(-3/2)
+    double ln_uK;                    // ln(U_K / U_{K-1})
     int K, L, n_T;
-    long long n_pairs;
+    int t_chunk;                     // temperatures of one block
+    int closed;                      // the closed form is allowed (ranges of kT and U)
+    // per temperature: [K][K] weights of the whole pieces at and above knot j, [K] exp(-(U_K - U_j)/kT),
+    // the tail's Chebyshev coefficients
+    const double *tab;
 };
+
+// doubles of A.tab per temperature
+__host__ __device__ constexpr int rate_tab_stride(int K) { return K * K + K + kRateCheb; }
 
 // Gamma(s, x) e^x for 1 <= s <= 2, x > 0.  Below x = s + 1 the power series of the lower
 // function gamma(s, x) = x^s e^-x sum_n x^n / (s (s+1) ... (s+n)) (Abramowitz & Stegun 6.5.29)
@@ -82,46 +104,12 @@ __device__ double upper_gamma_scaled(double s, double x)
     return pow(x, s) * f;
 }
 
-__global__ void k_rate_sym(const double *sigma, const double *g, int K, int L, double *out)
+// int sigma~ U exp(-(U - u0)/kT) dU by quadrature, piece by piece in increasing U (y, M: the knot values
+// and second derivatives of this thread's pair, `st` doubles apart)
+__device__ __noinline__ double rate_quadrature(const RateArgs &A, const double *y, const double *M, int st, double ymax,
+                                               double u0, double th, double ith)
 {
-    const long long n = (long long)K * L * L;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(i % L), a = (int)((i / L) % L);
-        const long long k = i / ((long long)L * L);
-        out[i] = 0.5 * (g[a] * sigma[i] + g[b] * sigma[(k * L + b) * L + a]);
-    }
-}
-
-__global__ void __launch_bounds__(128) k_rates(const __grid_constant__ RateArgs A, const double *sigma,
-                                                const double *g, const double *E, double *rate)
-{
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= A.n_pairs * A.n_T) return;
-    // temperature is the slow index: the lanes of a warp share kT and so take similar panel counts
-    const int t = (int)(i / A.n_pairs);
-    const long long q = i % A.n_pairs;
-    // q = b (b + 1) / 2 + a with a <= b
-    long long b = (long long)((sqrt(8.0 * (double)q + 1.0) - 1.0) * 0.5);
-    while (b * (b + 1) / 2 > q) --b;
-    while ((b + 1) * (b + 2) / 2 <= q) ++b;
-    const int ib = (int)b, ia = (int)(q - b * (b + 1) / 2);
-    const int K = A.K, L = A.L;
-    const double ga = g[ia], gb = g[ib];
-    double y[kRateMaxK], M[kRateMaxK];
-    double ymax = 0.0;
-    for (int k = 0; k < K; ++k) {
-        const size_t base = (size_t)k * L * L;
-        y[k] = 0.5 * (ga * sigma[base + (size_t)ia * L + ib] + gb * sigma[base + (size_t)ib * L + ia]);
-        ymax = fmax(ymax, fabs(y[k]));
-    }
-    for (int k = 0; k < K; ++k) {
-        double m = 0.0;
-        for (int j = 0; j < K; ++j) m = fma(A.Q[k][j], y[j], m);
-        M[k] = m;
-    }
-    const double th = A.kT[t], ith = 1.0 / th;
-    const double dE = E[ib] - E[ia], u0 = 0.5 * fabs(dE);
-    // acc = int sigma~ U exp(-(U - u0)/kT) dU, piece by piece in increasing U
+    const int K = A.K;
     double acc = 0.0;
     bool done = false;
     auto piece = [&](double lo, double hi, int kind, int k) {
@@ -133,6 +121,7 @@ __global__ void __launch_bounds__(128) k_rates(const __grid_constant__ RateArgs 
         const double h = kind ? A.u[k + 1] - A.u[k] : 0.0;
         // reciprocals once per piece (an FP64 division costs ~10 FMA slots on this GPU's FP64 pipe)
         const double ih = kind ? 1.0 / h : 0.0, iramp = kind ? 0.0 : y[0] / (A.u[0] - u0);
+        const double y0 = y[k * st], y1 = kind ? y[(k + 1) * st] : 0.0, M0 = M[k * st], M1 = kind ? M[(k + 1) * st] : 0.0;
         const double h26 = h * h * (1.0 / 6.0);
         // exp(-(U - u0)/kT) = exp(-(c - u0)/kT) exp(-(hp/2) x_j / kT): the node factors are the same
         // for every panel of the piece
@@ -154,8 +143,8 @@ __global__ void __launch_bounds__(128) k_rates(const __grid_constant__ RateArgs 
                 if (kind == 0) {
                     v = (U - u0) * iramp;
                 } else {
-                    const double tt = (U - A.u[k]) * ih, st = 1.0 - tt;
-                    v = st * y[k] + tt * y[k + 1] + h26 * ((st * st * st - st) * M[k] + (tt * tt * tt - tt) * M[k + 1]);
+                    const double tt = (U - A.u[k]) * ih, sr = 1.0 - tt;
+                    v = sr * y0 + tt * y1 + h26 * ((sr * sr * sr - sr) * M0 + (tt * tt * tt - tt) * M1);
                     v = fmax(v, 0.0);
                 }
                 s = fma(A.gw[j], v * U * (ec * ef[j]), s);
@@ -168,21 +157,151 @@ __global__ void __launch_bounds__(128) k_rates(const __grid_constant__ RateArgs 
     {
         // tail: y_K U_K^-p int_a^inf U^(1+p) exp(-(U - u0)/kT) dU
         //     = y_K U_K^-p kT^s [Gamma(s, a/kT) e^(a/kT)] exp(-(a - u0)/kT),  s = 2 + p
-        const double a = fmax(A.u[K - 1], u0), yK = y[K - 1], yJ = y[K - 2];
+        const double a = fmax(A.u[K - 1], u0), yK = y[(K - 1) * st], yJ = y[(K - 2) * st];
         double p = 0.0;
-        if (yK > 0.0 && yJ > 0.0) p = fmin(0.0, fmax(-1.0, log(yK / yJ) / log(A.u[K - 1] / A.u[K - 2])));
+        if (yK > 0.0 && yJ > 0.0) p = fmin(0.0, fmax(-1.0, log(yK / yJ) / A.ln_uK));
         if (yK != 0.0 && !done) {
             const double s = 2.0 + p, x = a * ith;
             acc += yK * pow(A.u[K - 1], -p) * pow(th, s) * upper_gamma_scaled(s, x) * exp(-(a - u0) * ith);
         }
     }
-    const double c = A.pref * pow(th, -1.5) * acc;
-    // exp(-dE/(2kT)) exp(-u0/kT): exp(-dE/kT) for an excitation, 1 for a quenching
-    const double ab = c * exp(-(0.5 * dE + u0) * ith) / ga;
-    const double ba = c * exp((0.5 * dE - u0) * ith) / gb;
-    const size_t plane = (size_t)t * L * L;
-    rate[plane + (size_t)ia * L + ib] = ab;
-    rate[plane + (size_t)ib * L + ia] = ba;
+    return acc;
+}
+
+// Lower incomplete gamma functions gamma(1..5, z) from ez = exp(-z).  z >= 2: upward recurrence
+// gamma(m + 1) = m gamma(m) - z^m e^-z (loses less than one digit there); below, the power series of
+// gamma(5, z) (Abramowitz & Stegun 6.5.29; 21 terms reach 1e-18 at z = 2) and the downward recurrence, all
+// of whose terms are positive.
+__device__ __forceinline__ void lower_gammas(double z, double ez, double G[5])
+{
+    const double z2 = z * z;
+    if (z >= 2.0) {
+        G[0] = 1.0 - ez;
+        G[1] = fma(-z, ez, G[0]);
+        G[2] = fma(2.0, G[1], -z2 * ez);
+        G[3] = fma(3.0, G[2], -z2 * z * ez);
+        G[4] = fma(4.0, G[3], -z2 * z2 * ez);
+    } else {
+        // sum_n z^n / (5 6 ... (5 + n)) = (1/5)(1 + z/6 (1 + z/7 (...)))
+        double s = 1.0;
+#pragma unroll
+        for (int n = 25; n >= 6; --n) s = fma(s, z * (1.0 / n), 1.0);
+        const double z4e = z2 * z2 * ez;
+        G[4] = 0.2 * s * z * z4e;
+        G[3] = 0.25 * (G[4] + z4e);
+        G[2] = (1.0 / 3.0) * (G[3] + z2 * z * ez);
+        G[1] = 0.5 * (G[2] + z2 * ez);
+        G[0] = fma(z, ez, G[1]);
+    }
+}
+
+// One thread per unordered pair (a <= b): the symmetrised cross sections of Eq. 20 (out, or NULL) and
+// both rates.  A block takes a tile of 16 x 8 pairs, so that the transposed reads sigma[k][a][b] of its
+// warps share 32-byte sectors.  Bound by the FP64 pipe: 1032 levels x 10 energies x 5 temperatures, all in
+// closed form, take 0.94 ms; the quadrature of every pair took 28.0 ms (one thread per pair and
+// temperature, a separate launch for the symmetrised cross sections).
+__global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant__ RateArgs A, const double *sigma,
+                                                         const double *g, const double *E, double *sym, double *rate)
+{
+    extern __shared__ double rsm[];
+    const int K = A.K, L = A.L;
+    const int a0 = blockIdx.x * kRateTa, b0 = blockIdx.y * kRateTb;
+    if (a0 > b0 + kRateTb - 1) return;
+    const int ia = a0 + threadIdx.x % kRateTa, ib = b0 + threadIdx.x / kRateTa;
+    if (ia >= L || ib >= L || ia > ib) return;
+    constexpr int st = kRateThreads;
+    double *y = rsm + threadIdx.x, *M = y + K * st;
+    const double ga = g[ia], gb = g[ib];
+    const size_t plane = (size_t)L * L, ab = (size_t)ia * L + ib, ba = (size_t)ib * L + ia;
+    const int t0 = blockIdx.z * A.t_chunk, t1 = min(A.n_T, t0 + A.t_chunk);
+    double ymax = 0.0;
+    for (int k = 0; k < K; ++k) {
+        const double v = 0.5 * (ga * sigma[k * plane + ab] + gb * sigma[k * plane + ba]);
+        y[k * st] = v;
+        ymax = fmax(ymax, fabs(v));
+        if (sym && t0 == 0) { sym[k * plane + ab] = v; sym[k * plane + ba] = v; }
+    }
+    for (int k = 0; k < K; ++k) {
+        double m = 0.0;
+        for (int j = 0; j < K; ++j) m = fma(A.Q[k][j], y[j * st], m);
+        M[k * st] = m;
+    }
+    const double dE = E[ib] - E[ia], u0 = 0.5 * fabs(dE);
+    // first knot at or above u0, and the Bernstein coefficients of the spline from there down to u0 (a NaN
+    // fails every comparison, so it takes the quadrature)
+    int j = 0;
+    while (j < K && !(A.u[j] >= u0)) ++j;
+    bool closed = A.closed && j < K && y[(K - 1) * st] >= 0.0 && y[0] >= 0.0;
+    for (int k = j > 0 ? j - 1 : 0; closed && k + 1 < K; ++k) {
+        const double h = A.u[k + 1] - A.u[k], h18 = h * h * (1.0 / 18.0);
+        const double ya = y[k * st], yb = y[(k + 1) * st], Ma = M[k * st], Mb = M[(k + 1) * st];
+        const double c1 = (2.0 * ya + yb) * (1.0 / 3.0) - h18 * (2.0 * Ma + Mb);
+        const double c2 = (ya + 2.0 * yb) * (1.0 / 3.0) - h18 * (Ma + 2.0 * Mb);
+        closed = ya >= 0.0 && yb >= 0.0 && c1 >= 0.0 && c2 >= 0.0;
+    }
+    const double iga = 1.0 / ga, igb = 1.0 / gb;
+    // quartic q of the cut piece (or the ramp): sigma~ U = sum_m q_m (U - u0)^m on [u0, U_j]
+    double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0, q4 = 0.0, w = 0.0, chx = 0.0;
+    if (closed) {
+        w = A.u[j] - u0;
+        if (j > 0) {
+            const int k = j - 1;
+            const double h = A.u[j] - A.u[k], ih = 1.0 / h, t = (u0 - A.u[k]) * ih, r = 1.0 - t;
+            const double ya = y[k * st], yb = y[j * st], Ma = M[k * st], Mb = M[j * st];
+            const double p0 = r * ya + t * yb + h * h * (1.0 / 6.0) * ((r * r * r - r) * Ma + (t * t * t - t) * Mb);
+            const double p1 = (yb - ya) * ih + h * (1.0 / 6.0) * ((1.0 - 3.0 * r * r) * Ma + (3.0 * t * t - 1.0) * Mb);
+            const double p2 = 0.5 * (r * Ma + t * Mb), p3 = (Mb - Ma) * ih * (1.0 / 6.0);
+            q0 = p0 * u0;
+            q1 = fma(p1, u0, p0);
+            q2 = fma(p2, u0, p1);
+            q3 = fma(p3, u0, p2);
+            q4 = p3;
+        } else if (w > 0.0) {
+            const double ramp = y[0] / w;
+            q1 = ramp * u0;
+            q2 = ramp;
+        }
+        // Chebyshev argument 2 p + 1 of the tail's exponent p in [-1, 0]
+        const double yK = y[(K - 1) * st], yJ = y[(K - 2) * st];
+        chx = 1.0;
+        if (yK > 0.0 && yJ > 0.0) chx = fma(2.0, fmin(0.0, fmax(-1.0, log(yK / yJ) / A.ln_uK)), 1.0);
+    }
+    for (int t = t0; t < t1; ++t) {
+        const double th = A.kT[t], ith = A.ikT[t];
+        double acc;
+        if (closed) {
+            const double *tab = A.tab + (size_t)t * rate_tab_stride(K);
+            // exp(-800) is zero in FP64, and z^4 exp(-z) with it
+            const double z = fmin(w * ith, 800.0), ez = exp(-z);
+            double G[5];
+            lower_gammas(z, ez, G);
+            acc = th * fma(q0, G[0], th * fma(q1, G[1], th * fma(q2, G[2], th * fma(q3, G[3], th * (q4 * G[4])))));
+            double whole = 0.0;
+            const double *W = tab + j * K;
+            for (int m = 0; m < K; ++m) whole = fma(__ldg(W + m), y[m * st], whole);
+            acc = fma(ez, whole, acc);
+            // tail: y_K kT U_K g(p) exp(-(U_K - u0)/kT), g(p) = x^-(1+p) Gamma(2 + p, x) e^x at x = U_K/kT;
+            // left out under the quadrature's remainder bound
+            const double eK = ez * __ldg(tab + K * K + j), uK = A.u[K - 1];
+            if (!(4.0 * ymax * th * (uK + th) * eK <= 1e-17 * acc)) {
+                const double *ch = tab + K * K + K;
+                double d1 = 0.0, d2 = 0.0;
+                for (int m = kRateCheb - 1; m > 0; --m) {
+                    const double d = fma(2.0 * chx, d1, __ldg(ch + m) - d2);
+                    d2 = d1;
+                    d1 = d;
+                }
+                acc = fma(y[(K - 1) * st] * th * uK * eK, fma(chx, d1, __ldg(ch) - d2), acc);
+            }
+        } else {
+            acc = rate_quadrature(A, y, M, st, ymax, u0, th, ith);
+        }
+        const double c = A.pref[t] * acc;
+        // exp(-dE/(2kT)) exp(-u0/kT): exp(-|dE|/kT) for an excitation, 1 for a quenching
+        const double ex = exp(-2.0 * u0 * ith);
+        rate[t * plane + ab] = c * (dE >= 0.0 ? ex : 1.0) * iga;
+        rate[t * plane + ba] = c * (dE >= 0.0 ? 1.0 : ex) * igb;
+    }
 }
 
 // Gauss-Legendre nodes and weights by Newton's iteration on P_n (three-term recurrence)
@@ -249,6 +368,101 @@ void natural_spline_map(const double *u, int K, double Q[kRateMaxK][kRateMaxK])
     }
 }
 
+// Gamma(s, x) e^x x^(1-s) for 1 <= s <= 2 and x > 0 (the series and the continued fraction of
+// upper_gamma_scaled)
+double upper_gamma_reduced(double s, double x)
+{
+    if (x < s + 1.0) {
+        double term = 1.0 / s, sum = term;
+        for (int n = 1; n < 300; ++n) {
+            term *= x / (s + n);
+            sum += term;
+            if (term < 1e-17 * sum) break;
+        }
+        return std::pow(x, 1.0 - s) * std::tgamma(s) * std::exp(x) - x * sum;
+    }
+    const double tiny = 1e-300;
+    double b = x + 1.0 - s, c = 1.0 / tiny, d = 1.0 / b, f = d;
+    for (int i = 1; i < 400; ++i) {
+        const double an = -i * (i - s);
+        b += 2.0;
+        d = an * d + b;
+        if (std::fabs(d) < tiny) d = tiny;
+        c = b + an / c;
+        if (std::fabs(c) < tiny) c = tiny;
+        d = 1.0 / d;
+        const double del = d * c;
+        f *= del;
+        if (std::fabs(del - 1.0) < 3e-16) break;
+    }
+    return x * f;
+}
+
+// gamma(1..5, z) on the host, as lower_gammas
+void host_gammas(double z, double G[5])
+{
+    const double ez = std::exp(-z);
+    if (z >= 8.0) {
+        G[0] = 1.0 - ez;
+        double zm = 1.0;
+        for (int m = 1; m < 5; ++m) {
+            zm *= z;
+            G[m] = m * G[m - 1] - zm * ez;
+        }
+        return;
+    }
+    double s = 1.0;
+    for (int n = 60; n >= 6; --n) s = 1.0 + s * z / n;
+    double zm = z * z * z * z;
+    G[4] = 0.2 * s * zm * z * ez;
+    for (int m = 4; m >= 1; --m) {
+        G[m - 1] = (G[m] + zm * ez) / m;
+        zm /= z;
+    }
+}
+
+// the closed form's tables (RateArgs::tab) of every temperature
+void rate_tables(const RateArgs &A, std::vector<double> &tab)
+{
+    const int K = A.K, stride = rate_tab_stride(K);
+    tab.assign((size_t)A.n_T * stride, 0.0);
+    const double pi = 3.14159265358979323846;
+    for (int t = 0; t < A.n_T; ++t) {
+        double *W = tab.data() + (size_t)t * stride, *eK = W + K * K, *ch = eK + K;
+        const double th = A.kT[t], uK = A.u[K - 1];
+        for (int j = 0; j < K; ++j) eK[j] = std::exp(-(uK - A.u[j]) / th);
+        // row j: pieces j .. K-2 relative to exp(-(U - U_j)/kT); row K-1 is zero
+        std::vector<double> row(K, 0.0);
+        for (int j = K - 2; j >= 0; --j) {
+            const double u = A.u[j], h = A.u[j + 1] - u, z = h / th, drop = std::exp(-z);
+            for (int m = 0; m < K; ++m) row[m] *= drop;
+            double G[5], I[6] = {0, 0, 0, 0, 0, 0};
+            host_gammas(z, G);
+            // I_m = int_0^h s^m exp(-s/kT) ds, then moments of t^m U = t^m (u + s), t = s/h
+            double pw = th, hm = 1.0, Tm[4];
+            for (int m = 0; m < 5; ++m) { I[m] = pw * G[m]; pw *= th; }
+            for (int m = 0; m < 4; ++m) { Tm[m] = (u * I[m] + I[m + 1]) / hm; hm *= h; }
+            // basis of the piece in t: y_a (1 - t), y_b t, h^2/6 [(r^3 - r) M_a + (t^3 - t) M_b], r = 1 - t
+            const double wya = Tm[0] - Tm[1], wyb = Tm[1];
+            const double wMa = h * h / 6.0 * (-2.0 * Tm[1] + 3.0 * Tm[2] - Tm[3]);
+            const double wMb = h * h / 6.0 * (Tm[3] - Tm[1]);
+            row[j] += wya;
+            row[j + 1] += wyb;
+            for (int m = 0; m < K; ++m) row[m] += wMa * A.Q[j][m] + wMb * A.Q[j + 1][m];
+            for (int m = 0; m < K; ++m) W[j * K + m] = row[m];
+        }
+        // Chebyshev series of g(p) on p in [-1, 0] (s = 2 + p), through its Chebyshev points
+        double f[kRateCheb];
+        for (int i = 0; i < kRateCheb; ++i)
+            f[i] = upper_gamma_reduced(1.5 + 0.5 * std::cos(pi * (i + 0.5) / kRateCheb), uK / th);
+        for (int m = 0; m < kRateCheb; ++m) {
+            double c = 0.0;
+            for (int i = 0; i < kRateCheb; ++i) c += f[i] * std::cos(pi * m * (i + 0.5) / kRateCheb);
+            ch[m] = c * (m ? 2.0 : 1.0) / kRateCheb;
+        }
+    }
+}
+
 bool rate_is_dev(const void *p)
 {
     if (!p) return false;
@@ -297,11 +511,23 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
     }
     natural_spline_map(A.u, K, A.Q);
     gauss_legendre(kGl, A.gx, A.gw);
-    A.pref = std::sqrt(8.0 / (3.14159265358979323846 * d->mu));
+    for (int t = 0; t < nT; ++t) {
+        A.ikT[t] = 1.0 / A.kT[t];
+        A.pref[t] = std::sqrt(8.0 / (3.14159265358979323846 * d->mu)) * std::pow(A.kT[t], -1.5);
+    }
     A.K = K;
     A.L = L;
     A.n_T = nT;
-    A.n_pairs = (long long)L * (L + 1) / 2;
+    A.ln_uK = std::log(A.u[K - 1] / A.u[K - 2]);
+    // the closed form's powers of kT stay far from the limits of FP64 in this range
+    A.closed = A.u[0] >= 1e-12 && A.u[K - 1] <= 1e6;
+    for (int t = 0; t < nT; ++t) A.closed = A.closed && A.kT[t] >= 1e-12 && A.kT[t] <= 1e6;
+    // one upload: degeneracies, level energies, tables
+    std::vector<double> up;
+    if (A.closed) rate_tables(A, up);
+    const size_t tab_n = up.size();
+    up.insert(up.end(), d->degeneracy, d->degeneracy + L);
+    up.insert(up.end(), d->level_energy, d->level_energy + L);
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     cudaError_t e;
@@ -314,7 +540,7 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
     auto cleanup = [&]() { for (void *p : tmp) cudaFreeAsync(p, st); };
     const size_t sig_bytes = sizeof(double) * (size_t)K * L * L, rate_bytes = sizeof(double) * (size_t)nT * L * L;
     const double *dsig = sigma;
-    double *dsym = sigma_sym, *drate = rate, *dgE = nullptr;
+    double *dsym = sigma_sym, *drate = rate, *dup = nullptr;
     const bool host_rate = !rate_is_dev(rate), host_sym = sigma_sym && !rate_is_dev(sigma_sym);
     if (!rate_is_dev(sigma)) {
         double *p;
@@ -325,24 +551,29 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
         }
         dsig = p;
     }
-    // degeneracies and level energies, one device buffer [g | E]; pageable copies are staged
-    // by the runtime before cudaMemcpyAsync returns
-    if ((e = get((void **)&dgE, sizeof(double) * 2 * (size_t)L)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(dgE, d->degeneracy, sizeof(double) * L, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(dgE + L, d->level_energy, sizeof(double) * L, cudaMemcpyHostToDevice, st)) != cudaSuccess) {
+    // a pageable copy is staged by the runtime before cudaMemcpyAsync returns
+    if ((e = get((void **)&dup, sizeof(double) * up.size())) != cudaSuccess ||
+        (e = cudaMemcpyAsync(dup, up.data(), sizeof(double) * up.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "staging levels");
     }
+    A.tab = dup;
+    const double *dg = dup + tab_n, *dE = dg + L;
     if (host_rate && (e = get((void **)&drate, rate_bytes)) != cudaSuccess) { cleanup(); return cuda_fail(e, "cudaMallocAsync"); }
     if (host_sym && (e = get((void **)&dsym, sig_bytes)) != cudaSuccess) { cleanup(); return cuda_fail(e, "cudaMallocAsync"); }
-    if (dsym) {
-        const long long n = (long long)K * L * L;
-        const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 16);
-        k_rate_sym<<<blocks, 256, 0, st>>>(dsig, dgE, K, L, dsym);
+    const int nta = (L + kRateTa - 1) / kRateTa, ntb = (L + kRateTb - 1) / kRateTb;
+    const size_t smem = sizeof(double) * 2 * (size_t)K * kRateThreads;
+    if ((e = cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) {
+        cleanup();
+        return cuda_fail(e, "cudaFuncSetAttribute");
     }
-    const long long work = A.n_pairs * nT;
-    k_rates<<<(unsigned)((work + 127) / 128), 128, 0, st>>>(A, dsig, dgE, dgE + L, drate);
-    count_launches(dsym ? 2 : 1);
+    // a thread runs all temperatures of its pair (the pair's spline is formed once); with too few tiles to
+    // fill the GPU the temperatures are spread over blocks instead
+    const long long tiles = (long long)nta * ntb / 2 + 1;
+    const int split = (int)std::min<long long>(nT, std::max<long long>(1, 608 / tiles));
+    A.t_chunk = (nT + split - 1) / split;
+    k_rates<<<dim3(nta, ntb, (nT + A.t_chunk - 1) / A.t_chunk), kRateThreads, smem, st>>>(A, dsig, dg, dE, dsym, drate);
+    count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) { cleanup(); return cuda_fail(e, "rate kernels"); }
     if (host_rate && (e = cudaMemcpyAsync(rate, drate, rate_bytes, cudaMemcpyDeviceToHost, st)) != cudaSuccess) {
         cleanup();
