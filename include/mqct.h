@@ -346,7 +346,7 @@ typedef struct {
                              non-zero entry; 0 everywhere = automatic (of the shapes every system
                              fits, the one with the most slots on the GPU that leaves two
                              trajectories per slot, else the one with the fewest slots; the
-                             (8,512) and (4,256) shapes first on ties).  1..7 = (slots per CTA at
+                             (4,256) and (8,512) shapes first on ties).  1..7 = (slots per CTA at
                              most, threads) of
                              (32,512) (16,512) (8,256) (8,512) (4,512) (16,256) (4,256); each system
                              gets the widest slot count (32, 16, 8 or 4, at most the shape's) its

@@ -2,28 +2,40 @@
 //
 // One CTA integrates B trajectories ("slots") at once; finished slots are refilled from the
 // device work queue, so trajectories of uneven length share a CTA.  Their phase-rotated stage
-// amplitudes form the N x B block C (one column per trajectory, FP32 complex, shared memory,
-// row-major: a row of four columns is 32 contiguous bytes).  The warps have two roles:
+// amplitudes form the N x B block C (FP32, shared memory, real and imaginary planes [row][slot], two
+// buffers by stage parity).  The warps have two roles:
 //
-//   element warps  own units (row r, 4 columns); per RK4 stage
-//     P3  contraction (Eq. 12): for every stored term l, Y_l = G^l C over the coalesced
-//         32-row sliced-ELL copy of G^l, combined per column with the FP32 spline values:
-//         w = M(R_b) c_b and u = M'(R_b) c_b; Coriolis stencil Dc = (J+ - J-) c; the stage
-//         derivative da/dt = -i exp(iEt) w + (dPhi/dt / 2) exp(iEt) Dc (Eq. 5) and the partial
-//         sums of the force -Re(c^dag u) (Eq. 9), the torque Re(c^dag D w) = -Re((Dc)^dag w)
-//         (Eq. 10) and, at stage 0, Re(c^dag w), |a|^2, E|a|^2, <J_y>;
-//     P4  RK4 accumulation and the next stage's input c (phase-rotated); the step update
-//         a + (dt/6) acc is compensated (two-sum), its rounding error carried into the next
+//   element warps  own units (row r, 4 slots) with their amplitudes (up to two units per thread) and RK4
+//     accumulators in registers; per RK4 stage
+//     contraction (Eq. 12): for every pair of stored terms, Y_l = G^l C over the row's non-zeros (one
+//         column and two values per entry, so a neighbour that both terms couple to is read once), folded
+//         with the FP32 spline values: w = M(R_b) c_b and u = M'(R_b) c_b;
+//     update: Coriolis stencil Dc = (J+ - J-) c, stage derivative da/dt = -i exp(iEt) w +
+//         (dPhi/dt / 2) exp(iEt) Dc (Eq. 5), RK4 accumulation and the next stage's input into the other
+//         C buffer; the partial sums of the force -Re(c^dag u) (Eq. 9), the torque
+//         Re(c^dag D w) = -Re((Dc)^dag w) (Eq. 10) and, at stage 0, Re(c^dag w), |a|^2, E|a|^2, <J_y>; the step
+//         update a + (dt/6) acc is compensated (two-sum), its rounding error carried into the next
 //         step's accumulator;
 //   slot warps     hold the FP64 classical state of the slots in registers, one lane per
 //     (component, slot): lane 8 c + j carries component c of (R, P_R, Phi, P_Phi) of slot j, so
-//     one FP64 instruction advances all four components of eight trajectories.  While the
-//     element warps contract stage s they look ahead: R of stage s+1 depends only on P_R of
-//     stage s, so its spline interval, 1/R and the spline values v_l, v_l' of stage s+1 are
-//     ready before stage s's force is known.  After the force and torque reductions only the
-//     RK4 update of (R, P_R, Phi, P_Phi) and dPhi/dt of the next stage remain (a handful of
-//     FP64 instructions); the bookkeeping of norm, total energy and P_Phi + <J_y>, the stop
-//     rule's outputs and the refill of a finished slot run during the next contraction.
+//     one FP64 instruction advances all four components of eight trajectories.
+//
+// One barrier per stage.  The slot warps are half a stage behind: while the element warps contract
+// stage s (whose spline values were looked ahead, since R of stage s depends only on P_R of stage
+// s-1), they sum the force and torque of stage s-1, advance the classical state and publish dPhi/dt
+// and the slots' states of stage s (an mbarrier that the element warps wait on between contraction and
+// update, by then long complete); then they look ahead to the spline values of stage s+1 and do the
+// bookkeeping of norm, total energy and P_Phi + <J_y>, the outputs and the refill of a finished slot.
+// Every chain of dependent FP64 instructions so runs beside the contraction.
+//
+// What bounds it: shared-memory reads of the neighbours' amplitudes (8 bytes per non-zero and slot) and
+// instruction issue.  Amplitude arithmetic is on packed pairs of slots (fma.rn.f32x2), which the planar
+// layout makes possible without moves; a unit's four slots are one 128-bit access per plane,
+// and consecutive rows of a warp are contiguous, so the accesses are free of bank conflicts but for the
+// borders of the m-blocks.  Measured (equal lengths, against two barriers per stage with scalar
+// arithmetic, interleaved complex C and one entry per term and column): N = 441, 1216 trajectories 42.8 -> 72 M
+// traj-steps/s, 2185 warp instructions per trajectory-stage (3974 before), issue slots 50 % busy,
+// shared-memory data path 66 %; N = 1600, 1216 trajectories 8.6 -> 16.3 M (its tables come from L2).
 //
 // Uneven batches (trajectories of several systems, i.e. basis sizes, in one call) run in this one
 // persistent launch: a CTA binds to a system (its share of the grid at the start is proportional
@@ -44,6 +56,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "tc_ptx.cuh"
 #include "traj_common.cuh"
 
 namespace mqct {
@@ -54,52 +67,110 @@ enum { SLOT_IDLE = 0, SLOT_ACTIVE = 1, SLOT_FINAL = 2, SLOT_WAIT = 3 };
 // slot warps for B slots (eight slots per warp, four component lanes per slot)
 __host__ __device__ constexpr int batch_slot_warps(int B) { return B > 8 ? B / 8 : 1; }
 
-struct F4x2 {  // four complex FP32 values (one unit row of four columns)
-    float2 v[4];
-};
-
-// Shared-memory layout of the [rows][B] float2 arrays (C, A, ACC, PHa, PHb): element e = row B + col
-// is stored at swz(e), which swaps the two 16-byte halves of a four-column unit when bit 3 of its
-// 16-byte chunk index is set.  Warps access units of consecutive rows (their own rows, and the
-// gathered neighbours of a banded coupling), whose 16-byte chunks would otherwise fall on only
-// half of the eight bank groups of a 128-byte line.
-__device__ __forceinline__ int swz(int e) { return e ^ (((e >> 4) & 1) << 1); }
-
-// the four columns e0 .. e0 + 3 (e0 a multiple of 4)
-__device__ __forceinline__ F4x2 ld4(const float2 *p, int e0)
+// ---- packed arithmetic on two slots (each half rounded as the scalar instruction)
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
 {
-    const float4 a = *reinterpret_cast<const float4 *>(p + swz(e0));
-    const float4 b = *reinterpret_cast<const float4 *>(p + swz(e0 + 2));
-    F4x2 r;
-    r.v[0] = make_float2(a.x, a.y); r.v[1] = make_float2(a.z, a.w);
-    r.v[2] = make_float2(b.x, b.y); r.v[3] = make_float2(b.z, b.w);
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+          "l"(reinterpret_cast<const unsigned long long &>(c)));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y)); }
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// one plane (real or imaginary parts) of a unit's four slots, as two packed pairs
+struct Q4 {
+    float2 p[2];
+};
+__device__ __forceinline__ Q4 neg4(const Q4 &a)
+{
+    Q4 r;
+    r.p[0] = neg2(a.p[0]);
+    r.p[1] = neg2(a.p[1]);
     return r;
 }
-
-__device__ __forceinline__ void st4(float2 *p, int e0, const F4x2 &r)
+__device__ __forceinline__ Q4 ldq(const float *p)
 {
-    *reinterpret_cast<float4 *>(p + swz(e0)) = make_float4(r.v[0].x, r.v[0].y, r.v[1].x, r.v[1].y);
-    *reinterpret_cast<float4 *>(p + swz(e0 + 2)) = make_float4(r.v[2].x, r.v[2].y, r.v[3].x, r.v[3].y);
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    Q4 r;
+    r.p[0] = make_float2(v.x, v.y);
+    r.p[1] = make_float2(v.z, v.w);
+    return r;
+}
+__device__ __forceinline__ void stq(float *p, const Q4 &r)
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(r.p[0].x, r.p[0].y, r.p[1].x, r.p[1].y);
+}
+__device__ __forceinline__ float qget(const Q4 &r, int j) { return (j & 1) ? r.p[j >> 1].y : r.p[j >> 1].x; }
+__device__ __forceinline__ void qset(Q4 &r, int j, float v)
+{
+    if (j & 1) r.p[j >> 1].y = v;
+    else r.p[j >> 1].x = v;
 }
 
-// per-slot values the element warps read during one stage, written by the slot warps during the
-// stage before (double-buffered by stage parity, so that writer and readers never overlap)
+// Sums over the lanes of a warp that share lane % G4 of eight values per lane (G4 in {1, 2, 4}): each
+// exchange halves the values a lane carries, so 15 shuffles or fewer take the place of 8 x 5.  On
+// return v[0] of the lane is the sum of the value whose index has bits (2, 1, 0) = lane bits (4, 3, 2).
+__device__ __forceinline__ float reduce8(float (&v)[8], int lane, int G4)
+{
+    const unsigned full = 0xffffffffu;
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float keep = h4 ? v[i + 4] : v[i], send = h4 ? v[i] : v[i + 4];
+        v[i] = keep + __shfl_xor_sync(full, send, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float keep = h3 ? v[i + 2] : v[i], send = h3 ? v[i] : v[i + 2];
+        v[i] = keep + __shfl_xor_sync(full, send, 8);
+    }
+    const float keep = h2 ? v[1] : v[0], send = h2 ? v[0] : v[1];
+    float x = keep + __shfl_xor_sync(full, send, 4);
+    if (G4 < 4) x += __shfl_xor_sync(full, x, 2);
+    if (G4 < 2) x += __shfl_xor_sync(full, x, 1);
+    return x;
+}
+
+// per-slot values the element warps read during one stage: vid, dvid are looked ahead (written during
+// the stage before), the others published during the stage (double-buffered by stage parity)
 template <int B>
 struct SlotView {
     __align__(16) float hp[B];    // dPhi/dt / 2 (FP32 view)
-    __align__(16) float dtf[B];   // dt (FP32 view)
+    __align__(16) float dtf[B], hdtf[B], h6f[B], ih6f[B];  // dt, dt/2, dt/6, 6/dt (FP32 views)
     __align__(16) float vid[B];   // sum of the identity terms' v_l (FP32 spline)
     __align__(16) float dvid[B];  // and of their v_l'
-    int state[B], traj[B], s0[B], steps[B];
+    __align__(16) int state[B];
+    __align__(16) int steps[B];
+    int traj[B], s0[B];
 };
 
 // per-slot values of the slot warps that are not needed at every stage (shared memory keeps
-// them out of the registers the element warps' stage derivatives need)
+// them out of the registers)
 struct SlotCold {
     double e0, j0, ndev, edev, jdev;  // initial E_tot and P_Phi + <J_y>, running deviations
     double last_dt, r_end, i2m0;      // dt of the phase increments; stop radius; (1/mu)/R^2 at stage 0
     int status, max_steps, traj, s0;
-    float dtf;
+    float dtf, ih6f;
 };
 
 // shared state of one CTA besides the big per-element arrays
@@ -108,19 +179,22 @@ struct BatchShared {
     DevSys S;
     SlotView<B> view[2];
     SlotCold cold[B];
-    float2 sum[6][B];  // cross-warp sums (hi, lo) of the six partial sums of the last phase B
-    int live;
-    int cur;           // system the CTA is bound to (-1: no work left)
+    int live[B > 8 ? B / 8 : 1];  // per slot warp: some slot of it is not idle (set at stage 0)
+    int cur;                      // system the CTA is bound to (-1: no work left)
+    int timeout;                  // a bounded wait ran out
+    __align__(8) uint64_t published;  // mbarrier: the slot warps have published a stage's views
 };
 
-// dynamic shared memory of a CTA bound to a system with B slots: inc [NL][B] (u64), C, A, ACC [n][B]
-// float2, PHa, PHb [NL][B] float2, vv, dvv [2][L][B] float, elev [NL] float, red [NE][B][8] float
-template <int BMAX, int T>
+constexpr long long kBatchWait = 1ll << 17;  // polls of at most ~1 us
+
+// dynamic shared memory of a CTA bound to a system with B slots: inc [NL][B] (u64), C [2][re, im][n][B], with more than
+// two units per thread the amplitudes [re, im][n][B], PHa, PHb [re, im][NL][B], vv, dvv [2][2 groups][B], red [NE][6][B], elev [NL] (float)
+template <int BMAX, int T, int kUpt>
 size_t batched_smem(const DevSys &h, int B)
 {
     constexpr int NE = T / 32 - batch_slot_warps(BMAX);
-    const size_t nl = h.n_levels, n = h.n, L = h.L;
-    return 8 * nl * B + 8 * (3 * n * B + 2 * nl * B) + 4 * (4 * L * B + nl) + 4 * (size_t)NE * B * 8 + 16;
+    const size_t nl = h.n_levels, n = h.n, nv = 2 * h.n_grp;
+    return 8 * nl * B + 4 * ((kUpt <= 2 ? 4 : 6) * n * B + 4 * nl * B + 4 * nv * B + nl + (size_t)NE * 6 * B) + 16;
 }
 
 template <int T>
@@ -159,10 +233,10 @@ __device__ int pick_system(const BatchMultiArgs &a, bool first)
 }
 
 // everything a CTA does while bound to system `cur`: with BC > 0 its slot count is the compile-time
-// constant BC, with BC = 0 the system's entry of a.slots
+// constant BC, with BC = 0 the system's entry of a.slots; `phase` counts the stages published
 template <int BC, int BMAX, int T, int kUpt>
 __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchShared<BMAX> &sh, int cur,
-                                               unsigned char *smraw)
+                                               unsigned char *smraw, unsigned &phase)
 {
     static_assert(BC % 4 == 0 && BC <= BMAX, "slots per CTA");
     constexpr int NS = batch_slot_warps(BMAX);  // slot warps (the last NS warps)
@@ -170,47 +244,34 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
     constexpr int TE = NE * 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool slot_warp = warp >= NE;
-    const int sc = lane >> 3, sj = lane & 7;
-    const int sb = slot_warp ? 8 * (warp - NE) + sj : 0;
     const unsigned full = 0xffffffffu;
-    const unsigned m4 = 0x01010101u << sj;  // the four component lanes of this slot
     const DevSys &S = sh.S;
     const int B = BC > 0 ? BC : a.slots[cur];    // slots (4, 8, 16 or 32)
-    const int G4 = B / 4;                        // four-column groups per row
+    const int G4 = B / 4;                        // four-slot groups per row
     const int lg4 = G4 == 1 ? 0 : (G4 == 2 ? 1 : (G4 == 4 ? 2 : 3));
-    const int n = S.n, NL = S.n_levels, L = S.L;
+    const int n = S.n, NL = S.n_levels, L = S.L, ng = S.n_grp, NV = 2 * ng;
+    const int np = n * B;  // floats of one plane of C
     const int *order = a.lists + (size_t)cur * a.n;
     int *queue = a.queues + cur;
     const int count = a.counts ? a.counts[cur] : a.n;
-    unsigned long long *inc = reinterpret_cast<unsigned long long *>(smraw);
-    float2 *C = reinterpret_cast<float2 *>(inc + (size_t)NL * B);
-    float2 *A = C + (size_t)n * B, *ACC = A + (size_t)n * B;
-    float2 *PHa = ACC + (size_t)n * B, *PHb = PHa + (size_t)NL * B;
-    float *vv = reinterpret_cast<float *>(PHb + (size_t)NL * B), *dvv = vv + 2 * (size_t)L * B;
-    float *elev = dvv + 2 * (size_t)L * B;
-    float *red = elev + NL;  // [NE][B][8]
+    float *C = reinterpret_cast<float *>(smraw);           // [2][re, im][np]
+    [[maybe_unused]] float *Asm = C + 4 * np;              // [re, im][np] when the amplitudes are not in registers
+    float *PHa = C + (kUpt <= 2 ? 4 : 6) * np, *PHb = PHa + 2 * NL * B;  // [re, im][NL][B]
+    float *vv = PHb + 2 * NL * B, *dvv = vv + 2 * NV * B;  // [2][NV][B]
+    float *red = dvv + 2 * NV * B;                         // [NE][6][B]
+    unsigned long long *inc = reinterpret_cast<unsigned long long *>(red + NE * 6 * B);  // [NL][B]
+    float *elev = reinterpret_cast<float *>(inc + NL * B);
     for (int l = tid; l < NL; l += T) elev[l] = (float)S.lev_energy[l];
-    // columns of the slots that start at the first stage 0: e_s0, accumulators 0, phases of t = 0
-    // and t = dt/2 (after the slot warps' first claims; both roles share the work)
-    auto init_columns = [&]() {
-        for (int i = tid; i < n * B; i += T) {
-            const int r = i / B, bb = i % B;
-            const int st = sh.view[0].state[bb];
-            if (st != SLOT_ACTIVE && st != SLOT_FINAL) continue;
-            const float2 v = make_float2(r == sh.view[0].s0[bb] ? 1.0f : 0.0f, 0.0f);
-            A[swz(i)] = v; ACC[swz(i)] = make_float2(0.f, 0.f); C[swz(i)] = v;
-        }
-        for (int i = tid; i < NL * B; i += T) {
-            PHa[swz(i)] = make_float2(1.f, 0.f);
-            const int st = sh.view[0].state[i % B];
-            if (st == SLOT_ACTIVE || st == SLOT_FINAL) PHb[swz(i)] = phase_factor(inc[i], 1u);
-        }
-    };
-    if (tid == 0) sh.live = 1;
+    // spline-weight rows of groups of one term stay zero in their second half
+    for (int i = tid; i < 4 * NV * B; i += T) vv[i] = 0.f;
+    __syncthreads();
 
-    // The two roles run separate code with the same barriers (two per stage), so that the
+    // The two roles run separate code with the same barriers (one per stage), so that the
     // registers of one role are not kept alive in the other.
     if (slot_warp) {
+    const int sc = lane >> 3, sj = lane & 7;
+    const int sb = 8 * (warp - NE) + sj;
+    const unsigned m4 = 0x01010101u << sj;  // the four component lanes of this slot
     // slot-warp registers (lane 8 c + j: component c of (R, P_R, Phi, P_Phi) of slot 8 (warp - NE) + j)
     double q = 0.0, qs = 0.0, lacc = 0.0;
     double imu = 1.0 / S.mu, dtd = 1.0, hdt = 0.5, h6 = 1.0 / 6.0;
@@ -218,11 +279,12 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
     double ir_n = 0.1, i2m_n = 0.0;                   // look-ahead
     int steps = 0, state = SLOT_IDLE;
     bool below_n = false;
+    float2 bk = make_float2(0.f, 0.f);  // stage-0 sum of lane c: V, <J_y>, |a|^2, E|a|^2
 
     // Every lane of a slot warp runs the same instructions (lanes of slots >= B compute on copies
     // and store nothing), so that the shuffles between the four component lanes of a slot are
     // warp-uniform.
-    const bool slot_lane = slot_warp && sb < B;
+    const bool slot_lane = sb < B;
     const int sbc = sb < B ? sb : B - 1;   // a valid index for reads of the lanes past B
     SlotCold &cs = sh.cold[sbc];
     if (slot_lane && sc == 0) {
@@ -242,6 +304,9 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
             vw.s0[sb] = cs.s0;
             vw.steps[sb] = steps;
             vw.dtf[sb] = cs.dtf;
+            vw.hdtf[sb] = 0.5f * cs.dtf;
+            vw.h6f[sb] = cs.dtf * (1.0f / 6.0f);
+            vw.ih6f[sb] = cs.ih6f;
             vw.hp[sb] = (float)phid * 0.5f;
         }
     };
@@ -294,6 +359,7 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
                 cs.traj = t;
                 cs.s0 = s0;
                 cs.dtf = (float)tr.dt;
+                cs.ih6f = 6.0f / (float)tr.dt;
                 cs.r_end = tr.r_end;
                 cs.max_steps = tr.max_steps;
                 cs.status = 0;
@@ -302,14 +368,14 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
             }
             // fixed-point phase increments of every level for this dt (kept while dt repeats)
             if (new_dt)
-                for (int l = sc; l < NL; l += 4) inc[(size_t)l * B + sb] = phase_increment(S.lev_energy[l], tr.dt);
+                for (int l = sc; l < NL; l += 4) inc[l * B + sb] = phase_increment(S.lev_energy[l], tr.dt);
             __syncwarp(m4);
             return;
         }
     };
 
-    // look-ahead for stage s+1 (s = -1: a slot that starts at the next stage 0): R, its interval,
-    // 1/R and the spline values of every term, written to vv / dvv [(s+1) & 1]
+    // look-ahead for stage s+1 (s = -1: a slot that starts at the next stage 0): R, its interval and
+    // the spline values of every term, written to vv / dvv [(s+1) & 1]; then 1/R
     auto look_ahead = [&](int s) {
         const int par = (s + 1) & 1;
         const bool act = slot_lane && state == SLOT_ACTIVE;
@@ -321,20 +387,19 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
         int k;
         double x;
         locate_interval(S, Rn, k, x, below_n);
-        ir_n = 1.0 / Rn;
-        i2m_n = imu * ir_n * ir_n;
         const float xf = (float)x;
         float v0 = 0.f, d0 = 0.f;
         for (int l = sc; l < L; l += 4) {
             float v = 0.f, dv = 0.f;
             if (act || start) {
-                const float4 c = S.vcoef_f[(size_t)l * S.n_int + k];
+                const float4 c = __ldg(S.vcoef_f + (size_t)l * S.n_int + k);
                 v = fmaf(xf, fmaf(xf, fmaf(xf, c.w, c.z), c.y), c.x);
                 dv = fmaf(xf, fmaf(3.0f * xf, c.w, 2.0f * c.z), c.y);
             }
-            if (slot_lane) {
-                vv[((size_t)par * L + l) * B + sb] = v;
-                dvv[((size_t)par * L + l) * B + sb] = dv;
+            const int row = __ldg(S.grp_row + l);
+            if (slot_lane && row >= 0) {
+                vv[(par * NV + row) * B + sb] = v;
+                dvv[(par * NV + row) * B + sb] = dv;
             }
             if ((S.id_mask >> l) & 1ull) { v0 += v; d0 += dv; }
         }
@@ -346,15 +411,28 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
             sh.view[par].vid[sb] = v0;
             sh.view[par].dvid[sb] = d0;
         }
+        ir_n = 1.0 / Rn;
+        i2m_n = imu * ir_n * ir_n;
+    };
+
+    // compensated FP32 sum of quantity qq of this lane's slot over the element warps w0, w0 + dw, ...
+    auto wsum = [&](int qq, int w0, int dw) {
+        float hi = 0.f, lo = 0.f;
+#pragma unroll 4
+        for (int w2 = w0; w2 < NE; w2 += dw) {
+            float e2;
+            two_sum(hi, red[(w2 * 6 + qq) * B + sbc], hi, e2);
+            lo += e2;
+        }
+        return make_float2(hi, lo);
     };
 
     // total energy, P_Phi + <J_y> and norm of the state at the start of a step (or of the final
-    // state) from its stage-0 sums (sh.sum[2..5]): running maxima of their deviations, for the
-    // slots where `apply` holds
+    // state) from its stage-0 sums: running maxima of their deviations, for the slots where
+    // `apply` holds
     auto bookkeeping = [&](bool apply) {
-        const float2 pv = sh.sum[2 + sc][sbc];  // lane c converts V, |a|^2, E|a|^2, <J_y>
-        const double val = (double)pv.x + (double)pv.y;
-        const double V = comp(val, 0), NR = comp(val, 1), ER = comp(val, 2), JY = comp(val, 3);
+        const double val = (double)bk.x + (double)bk.y;
+        const double V = comp(val, 0), JY = comp(val, 1), NR = comp(val, 2), ER = comp(val, 3);
         const double PR = comp(q, 1), PP = comp(q, 3);
         const double et = 0.5 * (imu * PR * PR + PP * PP * cs.i2m0) + ER + V;
         const double jt = PP + 0.5 * JY;
@@ -370,9 +448,68 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
         __syncwarp();
     };
 
+    // the classical stage update from the sums of stage sp, the stop rule (sp = 3) and the start of
+    // waiting slots; afterwards state, dPhi/dt and 1/R are those of the next stage
+    auto advance = [&](int sp) {
+        // lanes c = 0, 1 sum the force, c = 2, 3 the torque, over half of the element warps each
+        float2 pv = wsum(sc >> 1, sc & 1, 2);
+        {
+            const float ohi = __shfl_xor_sync(full, pv.x, 8), olo = __shfl_xor_sync(full, pv.y, 8);
+            float hi, e2;
+            two_sum(pv.x, ohi, hi, e2);
+            pv = make_float2(hi, pv.y + olo + e2);
+        }
+        const double X2 = (double)pv.x + (double)pv.y;
+        const double pr = comp(qs, 1);
+        if (sp == 0 && slot_lane && sc == 0) cs.i2m0 = i2m;
+        const bool act = slot_lane && state == SLOT_ACTIVE;
+        const bool start = slot_lane && state == SLOT_WAIT && sp == 3;
+        {
+            // derivative l_c: (P_R / mu, F + P_Phi^2/(mu R^3), dPhi/dt, torque) (Eqs. 7-10)
+            const double X = sc == 0 ? pr : (sc == 2 ? phid : X2);
+            const double alpha = sc == 0 ? imu : 1.0, beta = sc == 1 ? t1 : 0.0;
+            double qs2 = qs, lacc2 = lacc;
+            stage_component(sp, alpha, X, beta, hdt, dtd, h6, q, qs2, lacc2);
+            if (act) { qs = qs2; lacc = lacc2; }
+        }
+        int add_status = 0;
+        if (sp == 3) {
+            const unsigned bad = __ballot_sync(full, act && !finite64(qs));
+            const double R = comp(qs, 0), PR = comp(qs, 1);
+            if (act) {
+                q = qs;
+                steps += 1;
+                if ((bad >> sj) & 0x01010101u) {
+                    add_status |= MQCT_TRAJ_NONFINITE;
+                    state = SLOT_FINAL;
+                } else if (ge_pos(R, cs.r_end) && __double_as_longlong(PR) > 0) {
+                    state = SLOT_FINAL;
+                } else if (steps >= cs.max_steps) {
+                    add_status |= MQCT_TRAJ_MAX_STEPS;
+                    state = SLOT_FINAL;
+                }
+            }
+        }
+        const double pp3 = comp(qs, 3);
+        if ((act && !(add_status & MQCT_TRAJ_NONFINITE)) || start) {
+            if (below_n) add_status |= MQCT_TRAJ_TABLE_RANGE;
+            ir = ir_n;
+            i2m = i2m_n;
+            phid = pp3 * i2m_n;
+        }
+        if (start) {
+            const int ms = cs.max_steps;
+            state = ms > 0 ? SLOT_ACTIVE : SLOT_FINAL;
+            if (ms <= 0) add_status |= MQCT_TRAJ_MAX_STEPS;
+        }
+        __syncwarp();
+        if (slot_lane && sc == 0 && add_status) cs.status |= add_status;
+    };
+
     // ---------------------------------------------------------------- start
     {
         if (slot_lane) claim();
+        __syncwarp();
         look_ahead(-1);
         if (slot_lane && state == SLOT_WAIT) {
             const int ms = cs.max_steps;
@@ -387,24 +524,44 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
         publish(0);
     }
     __syncthreads();
-    init_columns();
-    __syncthreads();
-    {
-        while (sh.live) {
-            for (int s = 0; s < 4; ++s) {
-                // ================================================================ phase A
-                {
-                // ---- slot warps during the contraction: bookkeeping of stage 0 (a finished slot
-                // at stage 1, before its refill; running slots at stage 2), the diagnostics and
-                // refill of a finished slot, then the look-ahead for stage s+1
+    __syncthreads();  // the element warps have set up the columns
+    bool run = true, first = true;
+    while (run) {
+        for (int s = 0; s < 4; ++s) {
+            // ---- while the element warps contract stage s: the classical stage from the sums of the
+            // stage before, and this stage's views
+            if (!first) {
+                advance((s + 3) & 3);
+                publish(s);
+            }
+            first = false;
+            if (s == 0) {
+                const unsigned live = __ballot_sync(full, slot_lane && state != SLOT_IDLE);
+                if (lane == 0) sh.live[warp - NE] = live != 0;
+                if (NS > 1) {
+                    asm volatile("bar.sync 1, %0;" ::"r"(NS * 32) : "memory");
+                    run = false;
+#pragma unroll
+                    for (int i = 0; i < NS; ++i) run |= sh.live[i] != 0;
+                } else {
+                    run = live != 0;
+                }
+            }
+            __syncwarp();
+            if (lane == 0) tc_mbar_arrive(&sh.published);
+            if (!run) break;
+            // ---- bookkeeping of stage 0 (a finished slot at stage 1, before its refill; running slots
+            // at stage 2), the diagnostics and refill of a finished slot, then the look-ahead
+            if (s == 1) {
+                bk = wsum(2 + sc, 0, 1);
                 const bool fin_any = __any_sync(full, slot_lane && state == SLOT_FINAL);
-                if (s == 1 && fin_any) {
+                if (fin_any) {
                     bookkeeping(slot_lane && state == SLOT_FINAL);
                     if (slot_lane && state == SLOT_FINAL) {
                         if (sc == 0) {
                             if (a.diag) {
                                 mqct_diag d;
-                                d.steps = steps; d.status = cs.status;
+                                d.steps = steps; d.status = cs.status | (sh.timeout ? MQCT_TRAJ_TIMEOUT : 0);
                                 d.norm_dev = cs.ndev; d.energy_dev = cs.edev; d.angmom_dev = cs.jdev;
                                 d.t_final = steps * dtd;
                                 a.diag[cs.traj] = d;
@@ -412,309 +569,353 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
                             if (a.t_done) a.t_done[cs.traj] = mqct_clock_ns();
                         }
                         __syncwarp(m4);
-                        claim();  // WAIT or IDLE: phases at stage 2, column at stage 3
+                        claim();  // WAIT or IDLE: phases and column at stage 3
                     }
+                    __syncwarp();
                 }
-                if (s == 2) bookkeeping(slot_lane && state == SLOT_ACTIVE);
-                const double pp3 = comp(qs, 3);
-                if (slot_lane && state == SLOT_ACTIVE) t1 = pp3 * phid * ir;  // P_Phi^2 / (mu R^3)
-                look_ahead(s);
-                }
-                __syncthreads();
-                // ================================================================ phase B
-                {
-                // ---- slot warps: cross-warp sums (compensated FP32), then the classical stage
-                const int nq = s == 0 ? 6 : 2;
-                const int sid = tid - TE;
-                for (int pidx = sid; pidx < nq * B; pidx += NS * 32) {
-                    const int qq = pidx / B, bb = pidx % B;
-                    float hi = 0.f, lo = 0.f;
-                    for (int w2 = 0; w2 < NE; ++w2) {
-                        float e2;
-                        two_sum(hi, red[((size_t)w2 * B + bb) * 8 + qq], hi, e2);
-                        lo += e2;
-                    }
-                    sh.sum[qq][bb] = make_float2(hi, lo);
-                }
-                if (NS > 1) asm volatile("bar.sync 1, %0;" ::"r"(NS * 32) : "memory");
-                else __syncwarp();
-                // lane c = 1 converts the force, c = 3 the torque (c = 0, 2: unused copies)
-                const float2 pv = sh.sum[sc == 3 ? 1 : 0][sbc];
-                const double X2 = (double)pv.x + (double)pv.y;
-                const double pr = comp(qs, 1);
-                if (s == 0 && slot_lane && sc == 0) cs.i2m0 = i2m;
-                const bool act = slot_lane && state == SLOT_ACTIVE;
-                const bool start = slot_lane && state == SLOT_WAIT && s == 3;
-                {
-                    // derivative l_c: (P_R / mu, F + P_Phi^2/(mu R^3), dPhi/dt, torque) (Eqs. 7-10)
-                    const double X = sc == 0 ? pr : (sc == 2 ? phid : X2);
-                    const double alpha = sc == 0 ? imu : 1.0, beta = sc == 1 ? t1 : 0.0;
-                    double qs2 = qs, lacc2 = lacc;
-                    stage_component(s, alpha, X, beta, hdt, dtd, h6, q, qs2, lacc2);
-                    if (act) { qs = qs2; lacc = lacc2; }
-                }
-                int add_status = 0;
-                if (s == 3) {
-                    const unsigned bad = __ballot_sync(full, act && !finite64(qs));
-                    const double R = comp(qs, 0), PR = comp(qs, 1);
-                    if (act) {
-                        q = qs;
-                        steps += 1;
-                        if ((bad >> sj) & 0x01010101u) {
-                            add_status |= MQCT_TRAJ_NONFINITE;
-                            state = SLOT_FINAL;
-                        } else if (ge_pos(R, cs.r_end) && __double_as_longlong(PR) > 0) {
-                            state = SLOT_FINAL;
-                        } else if (steps >= cs.max_steps) {
-                            add_status |= MQCT_TRAJ_MAX_STEPS;
-                            state = SLOT_FINAL;
-                        }
-                    }
-                }
-                const double pp3 = comp(qs, 3);
-                if ((act && !(add_status & MQCT_TRAJ_NONFINITE)) || start) {
-                    if (below_n) add_status |= MQCT_TRAJ_TABLE_RANGE;
-                    ir = ir_n;
-                    i2m = i2m_n;
-                    phid = pp3 * i2m_n;
-                }
-                if (start) {
-                    const int ms = cs.max_steps;
-                    state = ms > 0 ? SLOT_ACTIVE : SLOT_FINAL;
-                    if (ms <= 0) add_status |= MQCT_TRAJ_MAX_STEPS;
-                }
-                __syncwarp();
-                if (slot_lane && sc == 0 && add_status) cs.status |= add_status;
-                publish(s + 1);
-                if (s == 3) {
-                    const unsigned live = __ballot_sync(full, slot_lane && state != SLOT_IDLE);
-                    if (warp == NE && lane == 0) sh.live = 0;
-                    if (NS > 1) asm volatile("bar.sync 1, %0;" ::"r"(NS * 32) : "memory");
-                    if (lane == 0 && live) atomicOr(&sh.live, 1);
-                }
-                }
-                __syncthreads();
             }
+            look_ahead(s);
+            const double pp3 = comp(qs, 3);
+            if (slot_lane && state == SLOT_ACTIVE) t1 = pp3 * phid * ir;  // P_Phi^2 / (mu R^3)
+            if (s == 2) bookkeeping(slot_lane && state == SLOT_ACTIVE);
+            __syncthreads();
         }
     }
     } else {
-    __syncthreads();
-    init_columns();
-    __syncthreads();
     const int g = tid & (G4 - 1);
-    float2 kq[kUpt][4];  // stage derivative da/dt of the unit's four columns (Eq. 5)
-    while (sh.live) {
-        for (int s = 0; s < 4; ++s) {
-            const int par = s & 1;
-            const SlotView<BMAX> &vw = sh.view[par];
-            // ================================================================ phase A
-            {
-                // phase factors of the next distinct stage time: t + dt/2 (after stage 0) and
-                // t + dt (after stage 2); a slot that starts at the next stage 0 gets t = 0
-                if (s == 0 || s == 2) {
-                    float2 *dst = s == 0 ? PHb : PHa;
-                    for (int i = tid; i < NL * B; i += TE) {
-                        const int bb = i % B, st = vw.state[bb];
-                        if (st == SLOT_ACTIVE)
-                            dst[swz(i)] = phase_factor(inc[i], 2u * (unsigned)vw.steps[bb] + (s == 0 ? 1u : 2u));
-                        else if (st == SLOT_WAIT && s == 2)
-                            dst[swz(i)] = make_float2(1.f, 0.f);
-                    }
-                }
-                // ---- P3: contraction, derivative, partial sums
-                const float2 *PHc = (s == 0 || s == 3) ? PHa : PHb;
-                const float *vvs = vv + (size_t)par * L * B, *dvvs = dvv + (size_t)par * L * B;
-                int cst[4];
-                bool any = false;
+    // amplitudes and RK4 accumulators of the units' four slots in registers; with more than two units per
+    // thread the amplitudes in shared memory (own values only)
+    constexpr bool kRegA = kUpt <= 2;
+    Q4 Rx[kRegA ? kUpt : 1] = {}, Ry[kRegA ? kUpt : 1] = {}, Kx[kUpt], Ky[kUpt];
+    auto get_a = [&](int k, int o, Q4 &x, Q4 &y) {
+        if constexpr (kRegA) { x = Rx[k]; y = Ry[k]; }
+        else { x = ldq(Asm + o); y = ldq(Asm + np + o); }
+    };
+    auto set_a = [&](int k, int o, const Q4 &x, const Q4 &y) {
+        if constexpr (kRegA) { Rx[k] = x; Ry[k] = y; }
+        else { stq(Asm + o, x); stq(Asm + np + o, y); }
+    };
+    __syncthreads();
+    // columns of the slots that start at the first stage 0: e_s0, accumulators 0, phase of t = dt/2
+    bool any = false;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    cst[j] = vw.state[4 * g + j];
-                    any |= cst[j] == SLOT_ACTIVE || cst[j] == SLOT_FINAL;
-                }
-                float fp[4] = {0, 0, 0, 0}, tp[4] = {0, 0, 0, 0}, vp[4] = {0, 0, 0, 0};
-                float np_[4] = {0, 0, 0, 0}, ep[4] = {0, 0, 0, 0}, jp[4] = {0, 0, 0, 0};
-                const float4 hp4 = *reinterpret_cast<const float4 *>(vw.hp + 4 * g);
-                const float hp[4] = {hp4.x, hp4.y, hp4.z, hp4.w};
-                const float4 vi = *reinterpret_cast<const float4 *>(vw.vid + 4 * g);
-                const float4 dvi = *reinterpret_cast<const float4 *>(vw.dvid + 4 * g);
-                const float vi_[4] = {vi.x, vi.y, vi.z, vi.w}, dvi_[4] = {dvi.x, dvi.y, dvi.z, dvi.w};
+    for (int j = 0; j < 4; ++j) any |= sh.view[0].state[4 * g + j] != SLOT_IDLE;
 #pragma unroll
-                for (int k = 0; k < kUpt; ++k) {
-                    const int u = tid + k * TE, r = u >> lg4;
-                    if (r >= n || !any) continue;
-                    const F4x2 c = ld4(C, r * B + 4 * g);
-                    F4x2 w, uu;
+    for (int k = 0; k < kUpt; ++k) {
+        const int r = (tid + k * TE) >> lg4;
+        Q4 x, y;
+        Kx[k].p[0] = Kx[k].p[1] = Ky[k].p[0] = Ky[k].p[1] = y.p[0] = y.p[1] = make_float2(0.f, 0.f);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        w.v[j] = make_float2(vi_[j] * c.v[j].x, vi_[j] * c.v[j].y);
-                        uu.v[j] = make_float2(dvi_[j] * c.v[j].x, dvi_[j] * c.v[j].y);
-                    }
-                    const int sl = r >> 5, rl = r & 31;
-                    for (int f = 0; f < S.n_f; ++f) {
-                        const int *so = S.f_sl_off + (size_t)f * (S.n_slices + 1);
-                        const int o0 = __ldg(so + sl), o1 = __ldg(so + sl + 1);
-                        const int2 *pe = S.f_cvf + o0 + rl;
-                        const int width = (o1 - o0) >> 5;
-                        float2 y[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-#pragma unroll 2
-                        for (int e = 0; e < width; ++e, pe += kSlice) {
-                            const int2 cv = __ldg(pe);
-                            const int col = cv.x;
-                            const float gv = __int_as_float(cv.y);
-                            const F4x2 z = ld4(C, col * B + 4 * g);
+        for (int j = 0; j < 4; ++j)
+            qset(x, j, sh.view[0].state[4 * g + j] != SLOT_IDLE && r == sh.view[0].s0[4 * g + j] ? 1.0f : 0.0f);
+        if (r < n) {
+            set_a(k, r * B + 4 * g, x, y);
+            stq(C + r * B + 4 * g, x);
+            stq(C + np + r * B + 4 * g, y);
+        }
+    }
+    for (int i = tid; i < NL * B; i += TE) {
+        const float2 p = sh.view[0].state[i % B] != SLOT_IDLE ? phase_factor(inc[i], 1u) : make_float2(1.f, 0.f);
+        PHb[i] = p.x;
+        PHb[NL * B + i] = p.y;
+        PHa[i] = 1.f;  // t = 0
+        PHa[NL * B + i] = 0.f;
+    }
+    __syncthreads();
+
+    // one RK4 stage of this warp's units; false once no slot is live
+    auto stage = [&](auto s0c, int s) -> bool {
+        constexpr bool S0 = decltype(s0c)::value;
+        const int par = s & 1;
+        const SlotView<BMAX> &vw = sh.view[par];
+        const float *Cc = C + par * 2 * np + 4 * g;
+        float *Cn = C + (par ^ 1) * 2 * np + 4 * g;
+        const float *PHc = ((S0 || s == 3) ? PHa : PHb) + 4 * g, *PHn = ((S0 || s == 1) ? PHb : PHa) + 4 * g;
+        const float *vvs = vv + par * NV * B + 4 * g, *dvvs = dvv + par * NV * B + 4 * g;
+        bool act = any, regular = false;
+        // the views of this stage, which the slot warps publish during the contraction: every lane of the
+        // warp waits, and the warp converges again afterwards
+        auto wait = [&]() {
+            // (bounded; after one wait ran out the others return at once and the results carry the flag)
+            if (!*(volatile int *)&sh.timeout && !tc_mbar_wait(&sh.published, phase & 1u, kBatchWait)) sh.timeout = 1;
+            __syncwarp();
+            const int4 st4 = *reinterpret_cast<const int4 *>(vw.state + 4 * g);
+            regular = st4.x == SLOT_ACTIVE && st4.y == SLOT_ACTIVE && st4.z == SLOT_ACTIVE && st4.w == SLOT_ACTIVE;
+            if (S0) {
+                const int4 sp = *reinterpret_cast<const int4 *>(vw.steps + 4 * g);
+                regular = regular && sp.x > 0 && sp.y > 0 && sp.z > 0 && sp.w > 0;
+            }
+            act = st4.x != SLOT_IDLE || st4.y != SLOT_IDLE || st4.z != SLOT_IDLE || st4.w != SLOT_IDLE;
+        };
+        float2 f2[2], t2[2], v2[2], j2[2], m2[2];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                y[j].x = fmaf(gv, z.v[j].x, y[j].x);
-                                y[j].y = fmaf(gv, z.v[j].y, y[j].y);
+        for (int i = 0; i < 2; ++i) f2[i] = t2[i] = v2[i] = j2[i] = m2[i] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < kUpt; ++k) {
+            const int r = (tid + k * TE) >> lg4;
+            const bool on = r < n && any;
+            const int ro = r * B;
+            // ---- contraction
+            Q4 wx, wy, ux, uy;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) wx.p[i] = wy.p[i] = ux.p[i] = uy.p[i] = make_float2(0.f, 0.f);
+            if (on) {
+            const int sl = r >> 5;
+            const int o0 = __ldg(S.g_off + sl) + (r & 31);
+            const float2 *pv = S.g_val + o0;
+            const unsigned short *pc = S.g_col + o0;
+            const int *pw = S.g_width + sl * ng;
+            for (int gi = 0; gi < ng; ++gi) {
+                const int wd = __ldg(pw + gi), width = wd & 0xffff;
+                Q4 ax, ay, bx, by;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) ax.p[i] = ay.p[i] = bx.p[i] = by.p[i] = make_float2(0.f, 0.f);
+                const float *vr = vvs + 2 * gi * B, *dr = dvvs + 2 * gi * B;
+                // two entries at a time: their table and amplitude reads are in flight together
+                auto entries = [&](auto two) {
+                    auto one = [&](float2 gv, const Q4 &zx, const Q4 &zy) {
+                        const float2 ga = dup2(gv.x), gb = dup2(gv.y);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            ax.p[i] = fma2(ga, zx.p[i], ax.p[i]); ay.p[i] = fma2(ga, zy.p[i], ay.p[i]);
+                            if constexpr (decltype(two)::value) {
+                                bx.p[i] = fma2(gb, zx.p[i], bx.p[i]); by.p[i] = fma2(gb, zy.p[i], by.p[i]);
                             }
                         }
-                        const int l = __ldg(S.f_term + f);
-                        const float4 v4 = *reinterpret_cast<const float4 *>(vvs + l * B + 4 * g);
-                        const float4 d4 = *reinterpret_cast<const float4 *>(dvvs + l * B + 4 * g);
-                        const float vl[4] = {v4.x, v4.y, v4.z, v4.w}, dl[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            w.v[j].x = fmaf(vl[j], y[j].x, w.v[j].x); w.v[j].y = fmaf(vl[j], y[j].y, w.v[j].y);
-                            uu.v[j].x = fmaf(dl[j], y[j].x, uu.v[j].x); uu.v[j].y = fmaf(dl[j], y[j].y, uu.v[j].y);
-                        }
+                    };
+                    int e = width;
+                    for (; e >= 2; e -= 2) {
+                        const float2 g0 = __ldg(pv), g1 = __ldg(pv + kSlice);
+                        const float *z0 = Cc + __ldg(pc) * B, *z1 = Cc + __ldg(pc + kSlice) * B;
+                        const Q4 x0 = ldq(z0), y0 = ldq(z0 + np), x1 = ldq(z1), y1 = ldq(z1 + np);
+                        pv += 2 * kSlice;
+                        pc += 2 * kSlice;
+                        one(g0, x0, y0);
+                        one(g1, x1, y1);
                     }
-                    const float au = __ldg(S.aupf + r), ad = __ldg(S.adnf + r);
-                    const F4x2 cu = ld4(C, __ldg(S.up + r) * B + 4 * g);
-                    const F4x2 cd = ld4(C, __ldg(S.dn + r) * B + 4 * g);
-                    const int lev = __ldg(S.lev + r);
-                    const F4x2 p = ld4(PHc, lev * B + 4 * g);
-                    F4x2 a0;
-                    if (s == 0) a0 = ld4(A, r * B + 4 * g);
-                    const float el = elev[lev];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 dc = make_float2(ad * cd.v[j].x - au * cu.v[j].x, ad * cd.v[j].y - au * cu.v[j].y);
-                        const float2 wj = w.v[j], pj = p.v[j];
-                        fp[j] -= c.v[j].x * uu.v[j].x + c.v[j].y * uu.v[j].y;
-                        tp[j] -= dc.x * wj.x + dc.y * wj.y;
-                        // conj(p) Dc = (J+ - J-) a at this stage (partners share the level energy)
-                        const float2 da = make_float2(pj.x * dc.x + pj.y * dc.y, pj.x * dc.y - pj.y * dc.x);
-                        kq[k][j].x = fmaf(hp[j], da.x, pj.x * wj.y - pj.y * wj.x);
-                        kq[k][j].y = fmaf(hp[j], da.y, -(pj.x * wj.x + pj.y * wj.y));
-                        if (s == 0) {
-                            const float2 aj = a0.v[j];
-                            const float pp = aj.x * aj.x + aj.y * aj.y;
-                            vp[j] += c.v[j].x * wj.x + c.v[j].y * wj.y;
-                            np_[j] += pp;
-                            ep[j] += el * pp;
-                            jp[j] += aj.x * da.y - aj.y * da.x;
-                        }
-                    }
-                }
-                // per-column sums over the warp (lanes of one column group), FP32; six quantities
-                // at stage 0, two (force, torque) at the others
-                auto warp_sums = [&](auto nqc) {
-                    constexpr int NQ = decltype(nqc)::value;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        float part[NQ];
-                        part[0] = fp[j];
-                        part[1] = tp[j];
-                        if constexpr (NQ == 6) {
-                            part[2] = vp[j]; part[3] = np_[j]; part[4] = ep[j]; part[5] = jp[j];
-                        }
-#pragma unroll
-                        for (int qq = 0; qq < NQ; ++qq) {
-                            float v = part[qq];
-#pragma unroll
-                            for (int off = G4; off < 32; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                            part[qq] = v;
-                        }
-                        if (lane < G4)
-#pragma unroll
-                            for (int qq = 0; qq < NQ; ++qq) red[((size_t)warp * B + 4 * lane + j) * 8 + qq] = part[qq];
+                    if (e) {
+                        const float2 g0 = __ldg(pv);
+                        const float *z0 = Cc + __ldg(pc) * B;
+                        const Q4 x0 = ldq(z0), y0 = ldq(z0 + np);
+                        pv += kSlice;
+                        pc += kSlice;
+                        one(g0, x0, y0);
                     }
                 };
-                if (s == 0) warp_sums(std::integral_constant<int, 6>{});
-                else warp_sums(std::integral_constant<int, 2>{});
+                if (wd >> 16) {
+                    entries(std::true_type{});
+                    const Q4 v = ldq(vr + B), d = ldq(dr + B);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        wx.p[i] = fma2(v.p[i], bx.p[i], wx.p[i]); wy.p[i] = fma2(v.p[i], by.p[i], wy.p[i]);
+                        ux.p[i] = fma2(d.p[i], bx.p[i], ux.p[i]); uy.p[i] = fma2(d.p[i], by.p[i], uy.p[i]);
+                    }
+                } else {
+                    entries(std::false_type{});
+                }
+                const Q4 v = ldq(vr), d = ldq(dr);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    wx.p[i] = fma2(v.p[i], ax.p[i], wx.p[i]); wy.p[i] = fma2(v.p[i], ay.p[i], wy.p[i]);
+                    ux.p[i] = fma2(d.p[i], ax.p[i], ux.p[i]); uy.p[i] = fma2(d.p[i], ay.p[i], uy.p[i]);
+                }
             }
-            __syncthreads();
-            // ================================================================ phase B
+            }
+            if (k == 0) wait();
+            // ---- update
+            if (!on) continue;
+            // identity terms
+            const Q4 cx = ldq(Cc + ro), cy = ldq(Cc + np + ro);
             {
-                // ---- P4: RK4 accumulation and the next stage's input (own units only)
-                const float2 *PHn = (s == 0 || s == 1) ? PHb : PHa;
-                const float4 dt4 = *reinterpret_cast<const float4 *>(vw.dtf + 4 * g);
-                const float dtj[4] = {dt4.x, dt4.y, dt4.z, dt4.w};
-                int cst[4];
-                bool all_act = true;
+                const Q4 vi = ldq(vw.vid + 4 * g), dvi = ldq(vw.dvid + 4 * g);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    wx.p[i] = fma2(vi.p[i], cx.p[i], wx.p[i]); wy.p[i] = fma2(vi.p[i], cy.p[i], wy.p[i]);
+                    ux.p[i] = fma2(dvi.p[i], cx.p[i], ux.p[i]); uy.p[i] = fma2(dvi.p[i], cy.p[i], uy.p[i]);
+                }
+            }
+            const int4 ri = __ldg(S.row_info + r);
+            const float *cu = Cc + (ri.x & 0xffff) * B, *cd = Cc + (int)((unsigned)ri.x >> 16) * B;
+            const int lo = ri.y * B;
+            Q4 px = ldq(PHc + lo), py = ldq(PHc + NL * B + lo);
+            const float2 nau = dup2(-__int_as_float(ri.z)), ad = dup2(__int_as_float(ri.w));
+            Q4 dcx, dcy;
+            {
+                const Q4 ux_ = ldq(cu), uy_ = ldq(cu + np), dx_ = ldq(cd), dy_ = ldq(cd + np);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    dcx.p[i] = fma2(ad, dx_.p[i], mul2(nau, ux_.p[i]));
+                    dcy.p[i] = fma2(ad, dy_.p[i], mul2(nau, uy_.p[i]));
+                }
+            }
+            if (S0 && !regular) {
+                // the first stage of a trajectory is at t = 0, where every phase factor is 1
+                const int4 sp = *reinterpret_cast<const int4 *>(vw.steps + 4 * g);
+                const int spj[4] = {sp.x, sp.y, sp.z, sp.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (spj[j] == 0) { qset(px, j, 1.f); qset(py, j, 0.f); }
+            }
+            // the next stage's time differs from this one's at stages 0 and 2 only
+            const Q4 npy = neg4(py);
+            Q4 qx = px, qy = py, nqy = npy;
+            if (S0 || s == 2) { qx = ldq(PHn + lo); qy = ldq(PHn + NL * B + lo); nqy = neg4(qy); }
+            const Q4 hp = ldq(vw.hp + 4 * g), nhp = neg4(hp);
+            // dt/6, dt or dt/2
+            const Q4 hs = ldq((!S0 && s == 3 ? vw.h6f : (s == 2 ? vw.dtf : vw.hdtf)) + 4 * g), nhs = neg4(hs);
+            Q4 ih6;
+            if (!S0 && s == 3) ih6 = ldq(vw.ih6f + 4 * g);
+            Q4 nx, ny, Ax, Ay;  // the next stage's input; the amplitudes at the start of the step
+            get_a(k, ro + 4 * g, Ax, Ay);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                f2[i] = fma2(cx.p[i], ux.p[i], f2[i]); f2[i] = fma2(cy.p[i], uy.p[i], f2[i]);
+                t2[i] = fma2(dcx.p[i], wx.p[i], t2[i]); t2[i] = fma2(dcy.p[i], wy.p[i], t2[i]);
+                // k = conj(p) (-i w + (dPhi/dt / 2) Dc), the imaginary part carried negated (ny = -Im), so
+                // that no operand needs a sign change (packed instructions have none)
+                const float2 zx = fma2(hp.p[i], dcx.p[i], wy.p[i]), zy = fma2(nhp.p[i], dcy.p[i], wx.p[i]);
+                const float2 kx = fma2(npy.p[i], zy, mul2(px.p[i], zx));
+                const float2 ky = fma2(px.p[i], zy, mul2(py.p[i], zx));
+                const float2 ax = Ax.p[i], ay = Ay.p[i];
+                if (S0) {
+                    v2[i] = fma2(cx.p[i], wx.p[i], v2[i]); v2[i] = fma2(cy.p[i], wy.p[i], v2[i]);
+                    // <J_y>: Im(a^dag D a) = Im(c^dag D c), the phases of a level's states cancel
+                    j2[i] = fma2(cx.p[i], dcy.p[i], j2[i]); m2[i] = fma2(cy.p[i], dcx.p[i], m2[i]);
+                    // the accumulator enters the step holding the rounding error of the last update
+                    Kx[k].p[i] = add2(kx, Kx[k].p[i]);
+                    Ky[k].p[i] = add2(ky, Ky[k].p[i]);
+                } else {
+                    const float2 wg = dup2(s == 3 ? 1.0f : 2.0f);
+                    Kx[k].p[i] = fma2(wg, kx, Kx[k].p[i]);
+                    Ky[k].p[i] = fma2(wg, ky, Ky[k].p[i]);
+                }
+                float2 yx, yy;
+                if (!S0 && s == 3) {
+                    // compensated a + (dt/6) acc (two-sum): far from the collision the
+                    // interaction-picture amplitudes change by increments a plain FP32 add
+                    // would round away; the error is carried to the next accumulator
+                    auto step2 = [&](float2 a0, float2 &acc, float2 h, float2 ih) {
+                        const float2 b0 = mul2(h, acc);
+                        const float2 sum = add2(a0, b0);
+                        const float2 bb = sub2(sum, a0);
+                        const float2 er = add2(sub2(a0, sub2(sum, bb)), sub2(b0, bb));
+                        acc = mul2(er, ih);
+                        return sum;
+                    };
+                    yx = step2(ax, Kx[k].p[i], hs.p[i], ih6.p[i]);
+                    yy = step2(ay, Ky[k].p[i], nhs.p[i], neg2(ih6.p[i]));
+                    Ax.p[i] = yx;
+                    Ay.p[i] = yy;
+                } else {
+                    yx = fma2(hs.p[i], kx, ax);
+                    yy = fma2(nhs.p[i], ky, ay);
+                }
+                nx.p[i] = fma2(nqy.p[i], yy, mul2(qx.p[i], yx));
+                ny.p[i] = fma2(qx.p[i], yy, mul2(qy.p[i], yx));
+            }
+            if (!regular) {
+                // slots that are not running: their arithmetic above is discarded
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    cst[j] = vw.state[4 * g + j];
-                    all_act &= cst[j] == SLOT_ACTIVE;
-                }
-                const float wgt = (s == 1 || s == 2) ? 2.0f : 1.0f;
-#pragma unroll
-                for (int k = 0; k < kUpt; ++k) {
-                    const int u = tid + k * TE, r = u >> lg4;
-                    if (r >= n) continue;
-                    const int o = r * B + 4 * g;
-                    const int lev = __ldg(S.lev + r);
-                    F4x2 a0 = ld4(A, o), acc = ld4(ACC, o), cn;
-                    // the columns not updated below keep their input; when all four are running,
-                    // every column is written and the old row is not needed
-                    if (!all_act) cn = ld4(C, o);
-                    const F4x2 pn = ld4(PHn, lev * B + 4 * g);
-                    bool wr_a = false;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int stj = cst[j];
-                        if (stj == SLOT_WAIT) {
-                            if (s == 3) {
-                                const float2 v = make_float2(r == vw.s0[4 * g + j] ? 1.0f : 0.0f, 0.0f);
-                                a0.v[j] = v; acc.v[j] = make_float2(0.f, 0.f); cn.v[j] = v;
-                                wr_a = true;
-                            }
-                            continue;
-                        }
-                        if (stj != SLOT_ACTIVE && stj != SLOT_FINAL) continue;
-                        if (stj == SLOT_FINAL && s != 0) continue;
-                        const float2 kk = kq[k][j];
-                        const float2 aj = a0.v[j];
-                        if (s == 0) {
-                            if (stj == SLOT_FINAL) {
-                                const float pp = aj.x * aj.x + aj.y * aj.y;
-                                const size_t oo = (size_t)vw.traj[4 * g + j] * a.nmax + __ldg(S.perm + r);
-                                if (a.pop) a.pop[oo] = (double)pp;
-                                if (a.amp) { a.amp[2 * oo] = aj.x; a.amp[2 * oo + 1] = aj.y; }
-                                continue;
-                            }
-                            // the accumulator enters the step holding the rounding error of the last update
-                            acc.v[j] = make_float2(kk.x + acc.v[j].x, kk.y + acc.v[j].y);
-                        } else {
-                            acc.v[j].x = fmaf(wgt, kk.x, acc.v[j].x);
-                            acc.v[j].y = fmaf(wgt, kk.y, acc.v[j].y);
-                            if (s == 3) {
-                                // compensated a + (dt/6) acc (two-sum): far from the collision the
-                                // interaction-picture amplitudes change by increments a plain FP32 add
-                                // would round away; the error is carried to the next accumulator
-                                const float h6f = dtj[j] * (1.0f / 6.0f), ih6 = 6.0f / dtj[j];
-                                const float ix = h6f * acc.v[j].x, iy = h6f * acc.v[j].y;
-                                float sx, sy, ex, ey;
-                                two_sum(aj.x, ix, sx, ex);
-                                two_sum(aj.y, iy, sy, ey);
-                                a0.v[j] = make_float2(sx, sy);
-                                acc.v[j] = make_float2(ex * ih6, ey * ih6);
-                                const float2 qn = pn.v[j];
-                                cn.v[j] = make_float2(qn.x * sx - qn.y * sy, qn.x * sy + qn.y * sx);
-                                wr_a = true;
-                                continue;
-                            }
-                        }
-                        const float bn = s == 2 ? dtj[j] : 0.5f * dtj[j];
-                        const float2 yn = make_float2(fmaf(bn, kk.x, aj.x), fmaf(bn, kk.y, aj.y));
-                        const float2 qn = pn.v[j];
-                        cn.v[j] = make_float2(qn.x * yn.x - qn.y * yn.y, qn.x * yn.y + qn.y * yn.x);
+                    const int stj = vw.state[4 * g + j];
+                    if (S0 && stj == SLOT_FINAL) {
+                        const float fx = qget(Ax, j), fy = qget(Ay, j);
+                        const size_t oo = (size_t)vw.traj[4 * g + j] * a.nmax + __ldg(S.perm + r);
+                        if (a.pop) a.pop[oo] = (double)fmaf(fx, fx, fy * fy);
+                        if (a.amp) { a.amp[2 * oo] = fx; a.amp[2 * oo + 1] = fy; }
                     }
-                    if (wr_a) st4(A, o, a0);
-                    st4(ACC, o, acc);
-                    st4(C, o, cn);
+                    if (stj == SLOT_WAIT && !S0 && s == 3) {
+                        const float v = r == vw.s0[4 * g + j] ? 1.0f : 0.0f;
+                        qset(Ax, j, v); qset(Ay, j, 0.f);
+                        qset(Kx[k], j, 0.f); qset(Ky[k], j, 0.f);
+                        qset(nx, j, v); qset(ny, j, 0.f);
+                    }
                 }
             }
+            if (!S0 && s == 3) set_a(k, ro + 4 * g, Ax, Ay);
+            stq(Cn + ro, nx);
+            stq(Cn + np + ro, ny);
+        }
+        __syncwarp();
+        ++phase;
+        if (S0) {
+            bool run = false;
+#pragma unroll
+            for (int i = 0; i < NS; ++i) run |= sh.live[i] != 0;
+            if (!run) return false;
+        }
+        // phase factors of the stages ahead: t + dt once stage 0 has read those of t, the next step's half
+        // time once stage 2 has read this one's (t = 0 of a starting slot needs none)
+        if (!S0 && s != 2) {
+            float *dst = s == 1 ? PHa : PHb;
+            for (int i = tid; i < NL * B; i += TE) {
+                const int bb = i % B, stb = vw.state[bb];
+                if (stb == SLOT_ACTIVE || (stb == SLOT_WAIT && s == 3)) {
+                    const unsigned nh = stb == SLOT_WAIT ? 1u : 2u * (unsigned)vw.steps[bb] + (s == 1 ? 2u : 3u);
+                    const float2 p = phase_factor(inc[i], nh);
+                    dst[i] = p.x;
+                    dst[NL * B + i] = p.y;
+                }
+            }
+        }
+        __syncwarp();
+        // per-slot sums over the warp (lanes of one group), FP32; six quantities at stage 0, two
+        // (force, torque) at the others
+        float *rw = red + warp * 6 * B;
+        // quantities q0 and q0 + 1 from their packed pairs
+        auto warp_sums = [&](int q0, const float2 (&s0)[2], const float2 (&s1)[2]) {
+            float part[8] = {s0[0].x, s0[0].y, s0[1].x, s0[1].y, s1[0].x, s1[0].y, s1[1].x, s1[1].y};
+            if (G4 <= 4) {
+                const float x = reduce8(part, lane, G4);
+                const int idx = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                if ((lane & 3) == g) rw[(q0 + (idx >> 2)) * B + 4 * g + (idx & 3)] = x;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    part[i] += __shfl_xor_sync(full, part[i], 8);
+                    part[i] += __shfl_xor_sync(full, part[i], 16);
+                    if (lane < 8) rw[(q0 + (i >> 2)) * B + 4 * g + (i & 3)] = part[i];
+                }
+            }
+        };
+#pragma unroll
+        for (int i = 0; i < 2; ++i) { f2[i] = neg2(f2[i]); t2[i] = neg2(t2[i]); }
+        warp_sums(0, f2, t2);
+        if constexpr (S0) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) j2[i] = sub2(j2[i], m2[i]);
+            warp_sums(2, v2, j2);
+            // |a|^2 and E|a|^2 (their own pass: fewer sums live at once)
+            float2 n2[2], e2[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) n2[i] = e2[i] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < kUpt; ++k) {
+                const int r = (tid + k * TE) >> lg4;
+                if (r >= n || !any) continue;
+                Q4 Ax, Ay;
+                get_a(k, r * B + 4 * g, Ax, Ay);
+                const float2 el = dup2(elev[__ldg(S.row_info + r).y]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float2 pp = fma2(Ax.p[i], Ax.p[i], mul2(Ay.p[i], Ay.p[i]));
+                    n2[i] = add2(n2[i], pp);
+                    e2[i] = fma2(el, pp, e2[i]);
+                }
+            }
+            __syncwarp();
+            warp_sums(4, n2, e2);
+        }
+        any = act;
+        __syncwarp();
+        return true;
+    };
+    for (;;) {
+        if (!stage(std::true_type{}, 0)) break;
+        __syncthreads();
+#pragma unroll 1
+        for (int s = 1; s < 4; ++s) {
+            stage(std::false_type{}, s);
             __syncthreads();
         }
     }
@@ -731,6 +932,11 @@ __global__ void __launch_bounds__(T, batched_min_blocks<T>()) k_batched_f32(Batc
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ BatchShared<BMAX> sh;
     bool first = true;
+    unsigned phase = 0;  // stages published so far (parity of the mbarrier)
+    if (threadIdx.x == 0) {
+        sh.timeout = 0;
+        tc_mbar_init(&sh.published, batch_slot_warps(BMAX));
+    }
     for (;;) {
         // bind to a system
         if (threadIdx.x == 0) {
@@ -742,7 +948,7 @@ __global__ void __launch_bounds__(T, batched_min_blocks<T>()) k_batched_f32(Batc
         first = false;
         const int cur = sh.cur;
         if (cur < 0) break;
-        batched_system<EXACT ? BMAX : 0, BMAX, T, kUpt>(a, sh, cur, smraw);
+        batched_system<EXACT ? BMAX : 0, BMAX, T, kUpt>(a, sh, cur, smraw, phase);
         __syncthreads();  // both roles are done with this system before the CTA binds to the next
     }
 }
@@ -754,7 +960,7 @@ int batched_slots(const DevSys &h, size_t cap)
 {
     constexpr int TE = (T / 32 - batch_slot_warps(BMAX)) * 32;
     for (int b = BMAX; b >= 4; b >>= 1)
-        if ((size_t)h.n * (b / 4) <= (size_t)kUpt * TE && batched_smem<BMAX, T>(h, b) + sizeof(BatchShared<BMAX>) <= cap)
+        if ((size_t)h.n * (b / 4) <= (size_t)kUpt * TE && batched_smem<BMAX, T, kUpt>(h, b) + sizeof(BatchShared<BMAX>) <= cap)
             return b;
     return 0;
 }
@@ -770,7 +976,7 @@ cudaError_t launch_batched(BatchMultiArgs a, const std::vector<const DevSys *> &
         if (b == 0) return cudaErrorInvalidConfiguration;
         a.slots[i] = b;
         minb = std::min(minb, b);
-        smem = std::max(smem, batched_smem<BMAX, T>(*hs[i], b));
+        smem = std::max(smem, batched_smem<BMAX, T, kUpt>(*hs[i], b));
     }
     const bool exact = minb == BMAX;
     const void *kern = exact ? (const void *)k_batched_f32<BMAX, T, kUpt, true>
@@ -797,7 +1003,7 @@ template <int BMAX, int T, int kUpt>
 static int shape_slots_of(const DevSys &h, size_t cap, size_t *smem)
 {
     const int b = batched_slots<BMAX, T, kUpt>(h, cap);
-    if (smem) *smem = b ? batched_smem<BMAX, T>(h, b) + sizeof(BatchShared<BMAX>) : 0;
+    if (smem) *smem = b ? batched_smem<BMAX, T, kUpt>(h, b) + sizeof(BatchShared<BMAX>) : 0;
     return b;
 }
 
@@ -832,10 +1038,12 @@ int batched_width(const DevSys &h)
 // cannot balance the slots when there are too few.  The rule: the shape with the most slots on
 // the GPU (slots per CTA x CTAs per SM x SMs, the slot count of the narrowest system) that still
 // leaves two trajectories per slot, else the one with the fewest slots; ties go to the earlier
-// entry of kAutoOrder, which puts the eight-slots-per-SM shapes first.  -1: no shape fits.
+// entry of kAutoOrder, which puts the eight-slots-per-SM shapes first, two CTAs of four slots before one of
+// eight: their barriers do not stop each other (3072 trajectories of N = 441 and uneven length: 361 against
+// 387 ms; equal lengths 62.2 against 60.7 M traj-steps/s).  -1: no shape fits.
 int batched_auto_shape(const std::vector<const DevSys *> &hs, int n, int sms)
 {
-    static const int kAutoOrder[7] = {3, 6, 4, 0, 1, 5, 2};
+    static const int kAutoOrder[7] = {6, 3, 4, 0, 1, 5, 2};
     int best = -1, fewest = -1;
     long long best_slots = -1, fewest_slots = 0;
     for (int k = 0; k < 7; ++k) {

@@ -61,8 +61,15 @@ struct DevSys {
     const int *f_cols;
     const double *f_val;
     const float *f_valf;       // FP32 copy of f_val (mixed-precision systems)
-    const int2 *f_cvf;         // f_cols and f_valf interleaved: (column, FP32 value bits) per entry,
-                               // one 8-byte load per entry (mixed-precision systems)
+    // FP32 batched kernel: the stored terms in groups of one or two that share columns (grp_row), each
+    // slice's entries of all groups consecutive: the values of the two terms and their column
+    int n_grp;
+    const int *g_off;          // [n_slices] first entry of the slice in g_val and g_col
+    const int *g_width;        // [n_slices][n_grp] entries per row; bit 16 set when the group has two terms
+    const float2 *g_val;       // 32 entries (one per row of the slice) per step
+    const unsigned short *g_col;
+    const int *grp_row;        // [L] spline-weight row 2 group + (0, 1) of each term; -1: not stored
+    const int4 *row_info;      // [n] (up | dn << 16, level, ladder factors aup, adn as FP32 bits)
     // Batched mixed-precision paths: FP32 spline coefficients of v_lambda, ladder factors
     const float4 *vcoef_f;     // [L][n_int]
     const float *aupf, *adnf;  // [n] FP32 ladder factors

@@ -553,13 +553,97 @@ extern "C" mqct_status mqct_create_system(const mqct_system_desc *d, mqct_system
                 vf[i] = make_float4((float)vcoef[i].x, (float)vcoef[i].y, (float)vcoef[i].z, (float)vcoef[i].w);
             std::vector<float> aupf(aup.begin(), aup.end()), adnf(adn.begin(), adn.end());
             up_(fvalf, &D.f_valf);
-            std::vector<int2> fcv(fcols.size());
-            for (size_t i = 0; i < fcols.size(); ++i) {
-                int bits;
-                std::memcpy(&bits, &fvalf[i], sizeof bits);
-                fcv[i] = make_int2(fcols[i], bits);
+            if (d->precision == MQCT_FP32 && n <= 0xffff) {
+                // groups of two terms whose non-zeros share columns: pairs in the order of the
+                // entries they save, a pair only when its union has at most 3/4 of the entries of the two
+                const int nf = (int)fterm.size();
+                auto merged = [&](int fa, int fb, int r) {
+                    std::vector<int> c;
+                    for (auto &e2 : grows[fterm[fa]][r]) c.push_back(e2.c);
+                    if (fb >= 0)
+                        for (auto &e2 : grows[fterm[fb]][r]) c.push_back(e2.c);
+                    std::sort(c.begin(), c.end());
+                    c.erase(std::unique(c.begin(), c.end()), c.end());
+                    return c;
+                };
+                struct Pair { long long save; int a, b; };
+                std::vector<Pair> cand;
+                for (int fa = 0; fa < nf; ++fa)
+                    for (int fb = fa + 1; fb < nf; ++fb) {
+                        long long sum = 0, uni = 0;
+                        for (int r = 0; r < n; ++r) {
+                            // entries of a row are in ascending column order
+                            const auto &ea = grows[fterm[fa]][r], &eb = grows[fterm[fb]][r];
+                            size_t ia = 0, ib = 0, shared = 0;
+                            while (ia < ea.size() && ib < eb.size()) {
+                                if (ea[ia].c == eb[ib].c) { ++shared; ++ia; ++ib; }
+                                else if (ea[ia].c < eb[ib].c) ++ia;
+                                else ++ib;
+                            }
+                            sum += (long long)(ea.size() + eb.size());
+                            uni += (long long)(ea.size() + eb.size() - shared);
+                        }
+                        if (4 * uni <= 3 * sum) cand.push_back({sum - uni, fa, fb});
+                    }
+                std::stable_sort(cand.begin(), cand.end(), [](const Pair &x, const Pair &y) { return x.save > y.save; });
+                std::vector<int> mate(nf, -1);
+                for (auto &c : cand)
+                    if (mate[c.a] < 0 && mate[c.b] < 0) { mate[c.a] = c.b; mate[c.b] = c.a; }
+                std::vector<std::pair<int, int>> grp;
+                for (int f = 0; f < nf; ++f)
+                    if (mate[f] < 0 || mate[f] > f) grp.push_back({f, mate[f]});
+                D.n_grp = (int)grp.size();
+                std::vector<int> grow(L, -1), goff(n_slices), gwidth((size_t)n_slices * std::max<size_t>(1, grp.size()), 0);
+                std::vector<float2> gval;
+                std::vector<uint16_t> gcol;
+                auto value = [&](int f, int r, int c) -> float {
+                    if (f >= 0)
+                        for (auto &e2 : grows[fterm[f]][r])
+                            if (e2.c == c) return (float)e2.v;
+                    return 0.f;
+                };
+                auto put = [&](int c, float va, float vb) {
+                    gcol.push_back((uint16_t)c);
+                    gval.push_back(make_float2(va, vb));
+                };
+                for (size_t g = 0; g < grp.size(); ++g) {
+                    grow[fterm[grp[g].first]] = 2 * (int)g;
+                    if (grp[g].second >= 0) grow[fterm[grp[g].second]] = 2 * (int)g + 1;
+                }
+                for (int sl = 0; sl < n_slices; ++sl) {
+                    goff[sl] = (int)gval.size();
+                    for (size_t g = 0; g < grp.size(); ++g) {
+                        std::vector<std::vector<int>> cols(kSlice);
+                        size_t width = 0;
+                        for (int q = 0; q < kSlice && sl * kSlice + q < n; ++q) {
+                            cols[q] = merged(grp[g].first, grp[g].second, sl * kSlice + q);
+                            width = std::max(width, cols[q].size());
+                        }
+                        gwidth[(size_t)sl * grp.size() + g] = (int)width | (grp[g].second >= 0 ? 1 << 16 : 0);
+                        for (size_t k = 0; k < width; ++k)
+                            for (int q = 0; q < kSlice; ++q) {
+                                const int r = std::min(sl * kSlice + q, n - 1);
+                                if (k < cols[q].size())
+                                    put(cols[q][k], value(grp[g].first, r, cols[q][k]), value(grp[g].second, r, cols[q][k]));
+                                else
+                                    put(r, 0.f, 0.f);  // padding: the row itself, zero values
+                            }
+                    }
+                }
+                std::vector<int4> rinfo(n);
+                for (int r = 0; r < n; ++r) {
+                    int ub, db;
+                    std::memcpy(&ub, &aupf[r], sizeof ub);
+                    std::memcpy(&db, &adnf[r], sizeof db);
+                    rinfo[r] = make_int4((int)((unsigned)up[r] | ((unsigned)dn[r] << 16)), S.lev[r], ub, db);
+                }
+                up_(grow, &D.grp_row);
+                up_(goff, &D.g_off);
+                up_(gwidth, &D.g_width);
+                up_(gval, &D.g_val);
+                up_(gcol, &D.g_col);
+                up_(rinfo, &D.row_info);
             }
-            up_(fcv, &D.f_cvf);
             up_(aupf, &D.aupf);
             up_(adnf, &D.adnf);
             up_(vf, &D.vcoef_f);
