@@ -96,7 +96,6 @@ void set_error(const std::string &msg);
 const char *last_error_cstr();
 
 // arguments of the persistent FP64 launch (propagate.cu)
-constexpr int kPropThreads = 512;  // upper bound of the block size (register budget)
 struct PropArgs {
     const DevSys *sys;
     const mqct_traj *trajs;
@@ -112,8 +111,10 @@ struct PropArgs {
     int smem_lev;  // max n_levels over systems
     int adapt;     // some system uses adaptive steps: two more vectors of smem_n in shared memory
 };
+// launches it over pa.n trajectories; pa.nmax: the largest basis, maxlev: the most levels, adapt: some system
+// uses adaptive steps.  cudaErrorInvalidConfiguration: it does not fit on an SM
+cudaError_t launch_propagate(PropArgs pa, int maxlev, bool adapt, cudaStream_t st);
 #ifdef __CUDACC__
-__global__ void __launch_bounds__(kPropThreads) k_propagate_fp64(PropArgs a);
 // device clock in nanoseconds (the global timer every SM shares)
 __device__ __forceinline__ long long mqct_clock_ns()
 {

@@ -123,7 +123,7 @@ extern "C" mqct_status mqct_propagate_noalloc(const mqct_system *systems, int32_
     if (n_systems > kNoallocMaxSystems)
         return fail(MQCT_ERR_INVALID_ARG, "mqct_propagate_noalloc: more than 16 systems (size of its static scratch)");
     if (n < 0) return fail(MQCT_ERR_INVALID_ARG, "mqct_propagate_noalloc: n < 0");
-    int nmax = 0, maxlev = 0, max_slices = 0;
+    int nmax = 0, maxlev = 0;
     for (int i = 0; i < n_systems; ++i) {
         if (!systems[i]) return fail(MQCT_ERR_INVALID_ARG, "mqct_propagate_noalloc: NULL system");
         const DevSys &h = systems[i]->s.h;
@@ -133,7 +133,6 @@ extern "C" mqct_status mqct_propagate_noalloc(const mqct_system *systems, int32_
             return fail(MQCT_ERR_INVALID_ARG, "mqct_propagate_noalloc: systems differ in path");
         nmax = std::max(nmax, h.n);
         maxlev = std::max(maxlev, h.n_levels);
-        max_slices = std::max(max_slices, h.n_slices);
     }
     if (n == 0) return MQCT_OK;
     if (!trajs || !on_device(trajs)) return fail(MQCT_ERR_INVALID_ARG, "mqct_propagate_noalloc: trajs must be device memory");
@@ -153,26 +152,15 @@ extern "C" mqct_status mqct_propagate_noalloc(const mqct_system *systems, int32_
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "k_noalloc_setup launch");
 
-    const int maxw = kPropThreads / 32;
-    const int per = (max_slices + maxw - 1) / maxw;
-    const int nwarps = std::max(4, std::min(maxw, (max_slices + per - 1) / per));
-    const int threads = nwarps * 32;
     bool adapt = false;
     for (int i = 0; i < n_systems; ++i) adapt |= systems[i]->s.h.adapt_tol > 0.0;
-    const size_t smem = sizeof(double2) * ((adapt ? 8 : 6) * (size_t)nmax + 2 * (size_t)maxlev);
-    int sms = 0, per_sm = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if ((e = cudaFuncSetAttribute(k_propagate_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return cuda_fail(e, "cudaFuncSetAttribute (basis too large for shared memory)");
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_propagate_fp64, threads, smem)) != cudaSuccess)
-        return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    if (per_sm < 1) return fail(MQCT_ERR_UNSUPPORTED, "mqct_propagate_noalloc: kernel does not fit on an SM");
     PropArgs pa{};
     pa.sys = dsys; pa.trajs = trajs; pa.order = nullptr; pa.n = n; pa.n_systems = n_systems; pa.queue = queue;
-    pa.pop = final_pop; pa.amp = final_amp; pa.diag = diag; pa.nmax = nmax; pa.smem_n = nmax; pa.smem_lev = maxlev;
-    pa.adapt = adapt ? 1 : 0;
-    k_propagate_fp64<<<std::min(n, sms * per_sm), threads, smem, st>>>(pa);
-    count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "k_propagate_fp64 launch");
+    pa.pop = final_pop; pa.amp = final_amp; pa.diag = diag; pa.nmax = nmax;
+    if ((e = launch_propagate(pa, maxlev, adapt, st)) != cudaSuccess) {
+        if (e == cudaErrorInvalidConfiguration)
+            return fail(MQCT_ERR_UNSUPPORTED, "mqct_propagate_noalloc: kernel does not fit on an SM");
+        return cuda_fail(e, "k_propagate_fp64 launch (basis too large for shared memory?)");
+    }
     return MQCT_OK;
 }

@@ -288,6 +288,26 @@ extern "C" mqct_status mqct_create_system(const mqct_system_desc *d, mqct_system
         S.max_block = std::max<int>(S.max_block, (int)b.size());
         for (int s : b) S.perm.push_back(s);
     }
+    if (d->precision == MQCT_FP64) {
+        // FP64 systems: rows by descending number of coupled columns (of all terms together on the PLAIN
+        // path, per term on the factorised one), so that the rows of a slice are equally long: a padded
+        // entry costs the FP64 pipe as much as a non-zero (N = 441: 3296 entries against 3840, 3189 non-zeros)
+        std::vector<int> len(n, 0);
+        if (d->path == MQCT_PATH_PLAIN) {
+            std::vector<std::vector<int>> cols(n);
+            for (int l = 0; l < L; ++l)
+                for (const Trip &e : G[l])
+                    if (e.v != 0.0) cols[e.r].push_back(e.c);
+            for (int r = 0; r < n; ++r) {
+                std::sort(cols[r].begin(), cols[r].end());
+                len[r] = (int)(std::unique(cols[r].begin(), cols[r].end()) - cols[r].begin());
+            }
+        } else {
+            for (int l = 0; l < L; ++l)
+                for (const Trip &e : G[l]) len[e.r] += e.v != 0.0;
+        }
+        std::stable_sort(S.perm.begin(), S.perm.end(), [&](int x, int y) { return len[x] > len[y]; });
+    }
     S.inv.assign(n, 0);
     for (int i = 0; i < n; ++i) S.inv[S.perm[i]] = i;
     S.lev.resize(n);
