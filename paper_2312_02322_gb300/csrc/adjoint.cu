@@ -6,9 +6,8 @@
 // so each trajectory starts the reverse sweep from abar_s = 2 w_t dL/dsigma[g_t][level(s)] a_s.
 // One CTA per trajectory, the factorised coupling M(R) = sum_l v_l(R) G^l (Eq. 12):
 //   1. forward RK4 (the same map as mqct_propagate), a checkpoint of the state every K steps;
-//   2. for each segment, last first: recompute its states from the checkpoint, then reverse
-//      every step: recompute the four stage states and apply the vector-Jacobian product of
-//      f (Eqs. 5, 7-10) in reverse stage order:
+//   2. for each segment, last first: recompute its states and stage states from the checkpoint, then
+//      reverse every step: apply the vector-Jacobian product of f (Eqs. 5, 7-10) in reverse stage order:
 //        kbar4 = dt/6 lam,                 Ybar4 = J4^T kbar4
 //        kbar3 = dt/3 lam + dt   Ybar4,    Ybar3 = J3^T kbar3
 //        kbar2 = dt/3 lam + dt/2 Ybar3,    Ybar2 = J2^T kbar2
@@ -68,8 +67,10 @@ struct AdjArgs {
     const double *dLds;       // [n_groups][n_levels]
     int K;                    // checkpoint interval
     int max_ckpt;             // checkpoints that fit in a CTA's scratch
-    unsigned char *scratch;   // per CTA: (max_ckpt + K) * stride bytes
+    unsigned char *scratch;   // per CTA: max_ckpt * stride + K * seg_stride bytes
     size_t stride;            // bytes per stored state
+    size_t seg_stride;        // bytes per step of a segment: its state and, with `stages`, the stage states
+    int stages;               // the recomputed segment keeps Y2..Y4 of each step (no second recomputation)
     unsigned char *vec;       // per CTA: vec_bytes of global memory for the work vectors when they do
     size_t vec_bytes;         //   not fit in shared memory (nullptr: shared memory)
     double *theta_traj;       // [n][P] per-trajectory gradient
@@ -91,6 +92,7 @@ struct AdjCtl {
     double p_r0;
     double x;                      // offset of R in its spline interval
     int steps, status, item, t, kint;
+    int n_term, term_l[kAdjMaxL], term_f[kAdjMaxL];  // terms with a matrix: lambda, stored index (-1: identity)
 };
 
 template <class R>
@@ -226,8 +228,8 @@ __device__ void fwd_eval(const DevSys &S, double t, unsigned n_half, const typen
     __syncthreads();
     for (int r = tid; r < n; r += nt) m.C[r] = cmul<R>(m.PH[S.lev[r]], Ya[r]);
     __syncthreads();
-    R force = 0;
-    const R vid = c.vid, dvid = c.dvid;
+    R force = 0, torque = 0;
+    const R vid = c.vid, dvid = c.dvid, hp = c.hp;
     for (int sl = warp; sl < S.n_slices; sl += nw) {
         const int r = sl * kSlice + lane;
         const V c0 = r < n ? m.C[r] : Cx<R>::mk(0, 0);
@@ -248,19 +250,25 @@ __device__ void fwd_eval(const DevSys &S, double t, unsigned n_half, const typen
             w.x = fma(c.v[l], y.x, w.x); w.y = fma(c.v[l], y.y, w.y);
             u.x = fma(c.dv[l], y.x, u.x); u.y = fma(c.dv[l], y.y, u.y);
         }
-        if (r < n) {
+        if (r >= n) continue;
+        force -= c0.x * u.x + c0.y * u.y;
+        if constexpr (sizeof(R) == 8) {
+            // the whole stage in this pass: with Dc = (J+ - J-) c the torque is -Re((Dc)^dag w) and
+            // k = conj(p) (-i w + (dPhi/dt / 2) Dc) (the ladder partners share the phase factor)
+            const double au = S.aup[r], ad = S.adn[r];
+            const V cu = m.C[S.up[r]], cd = m.C[S.dn[r]], p = m.PH[S.lev[r]];
+            const V dc = Cx<R>::mk(ad * cd.x - au * cu.x, ad * cd.y - au * cu.y);
+            torque -= dc.x * w.x + dc.y * w.y;
+            m.K[r] = cconjmul<R>(p, Cx<R>::mk(fma(hp, dc.x, w.y), fma(hp, dc.y, -w.x)));
+        } else {
             m.W[r] = w;
-            force -= c0.x * u.x + c0.y * u.y;
         }
     }
+    if constexpr (sizeof(R) == 4) {
     __syncthreads();
-    const R hp = c.hp;
-    R torque = 0;
     for (int r = tid; r < n; r += nt) {
         const int ru = S.up[r], rd = S.dn[r];
-        R au, ad;
-        if constexpr (sizeof(R) == 8) { au = S.aup[r]; ad = S.adn[r]; }
-        else { au = S.aupf[r]; ad = S.adnf[r]; }
+        const R au = S.aupf[r], ad = S.adnf[r];
         const V w = m.W[r], wu = m.W[ru], wd = m.W[rd], z = m.C[r];
         const V Dw = Cx<R>::mk(ad * wd.x - au * wu.x, ad * wd.y - au * wu.y);
         torque += z.x * Dw.x + z.y * Dw.y;
@@ -271,6 +279,7 @@ __device__ void fwd_eval(const DevSys &S, double t, unsigned n_half, const typen
         k.x = fma(hp, Dy.x, p.x * w.y - p.y * w.x);
         k.y = fma(hp, Dy.y, -(p.x * w.x + p.y * w.y));
         m.K[r] = k;
+    }
     }
     const R vals[2] = {force, torque};
     block_sums<R>(vals, 2, c, wred);
@@ -283,12 +292,169 @@ __device__ void fwd_eval(const DevSys &S, double t, unsigned n_half, const typen
     __syncthreads();
 }
 
-// Vector-Jacobian product at stage (t, Y): given the cotangent (KB, c.kb) of f, add J^T kbar
-// to (YN, c.ynew) and the parameter cotangent to c.theta.  Needs terms_at(Y_R).
-template <class R>
-__device__ void vjp_eval(const DevSys &S, double t, unsigned n_half, const typename Cx<R>::T *Ya, const double *Yq,
-                         AdjSmem<R> &m, AdjCtl<R> &c, R *wred)
+// sums over the lanes of a warp of sixteen values per lane, halving what a lane carries at each exchange (16
+// additions instead of 16 x 5): on return the even lane 2 i holds value i
+__device__ __forceinline__ double reduce16(double (&v)[16], int lane)
 {
+    const unsigned full = 0xffffffffu;
+#pragma unroll
+    for (int o = 16, k = 8; o > 1; o >>= 1, k >>= 1) {
+        const bool h = lane & o;
+#pragma unroll
+        for (int i = 0; i < k; ++i) {
+            const double keep = h ? v[i + k] : v[i], send = h ? v[i] : v[i + k];
+            v[i] = keep + __shfl_xor_sync(full, send, o);
+        }
+    }
+    return v[0] + __shfl_xor_sync(full, v[0], 1);
+}
+
+// Vector-Jacobian product at stage (t, Y) in FP64: given the cotangent (KB, c.kb) of f, add J^T kbar to
+// (YN, c.ynew) and the parameter cotangent to c.theta.  Needs terms_at(Y_R).
+//
+// Bound by the FP64 pipe, so arranged for the fewest FP64 instructions: M z and M Dc (z = p kbar, Dc = (J+ - J-) c)
+// enter the result as conj(p) M (i z - PPhibar Dc) only and are contracted as that one vector; the sums
+// Re(kbar^dag (-i conj(p) M' c)), Re(c^dag M'' c) and Re((Dc)^dag M' c) follow from the per-term sums alpha, beta, gamma
+// that the parameters need anyway; those are reduced five terms at a time (reduce16).  N = 441, 128 trajectories,
+// with the forward stage in one pass and the kept stage states: 1169 -> 695 ms.  The mixed form below keeps the
+// order of its sums, and with it its bits.
+__device__ void vjp_eval64(const DevSys &S, double t, const double2 *Ya, const double *Yq, AdjSmem<double> &m,
+                           AdjCtl<double> &c, double *wred)
+{
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int n = S.n, L = S.L;
+    const double R_ = Yq[0], PP = Yq[3], mu = S.mu;
+    const double PRb = c.kb[1], PPb = c.kb[3];
+    if (tid == 0) c.hp = 0.5 * PP / (mu * R_ * R_);
+    phases<double>(S, t, 0u, m);
+    __syncthreads();
+    for (int r = tid; r < n; r += nt) {
+        const double2 p = m.PH[S.lev[r]];
+        m.C[r] = cmul<double>(p, Ya[r]);
+        m.Z[r] = cmul<double>(p, m.KB[r]);
+    }
+    __syncthreads();
+    double2 *Q = m.MZ;  // i z - PPhibar Dc
+    for (int r = tid; r < n; r += nt) {
+        const double au = S.aup[r], ad = S.adn[r];
+        const double2 cu = m.C[S.up[r]], cd = m.C[S.dn[r]], z = m.Z[r];
+        const double2 dc = make_double2(ad * cd.x - au * cu.x, ad * cd.y - au * cu.y);
+        m.DC[r] = dc;
+        Q[r] = make_double2(fma(-PPb, dc.x, -z.y), fma(-PPb, dc.y, z.x));
+    }
+    // per-term sums alpha_l = Re(kbar^dag (-i conj(p) G^l c)) = Re(z^dag (-i G^l c)), beta_l = -Re(c^dag G^l c),
+    // gamma_l = -Re((Dc)^dag G^l c) of this warp's rows at wt[4 + 3 l ..], Re(z^dag Dc) at wt[1]
+    double *wt = wred + warp * kAdjRed;
+    for (int i = lane; i < 4 + 3 * L; i += 32) wt[i] = 0.0;
+    __syncthreads();
+    for (int sl = warp; sl < S.n_slices; sl += nw) {
+        const int r = sl * kSlice + lane;
+        const bool in = r < n;
+        const double2 zero = make_double2(0.0, 0.0);
+        const double2 c0 = in ? m.C[r] : zero, z0 = in ? m.Z[r] : zero, d0 = in ? m.DC[r] : zero, q0 = in ? Q[r] : zero;
+        double2 w = zero, u = zero, mq = zero;
+        for (int t0 = 0; t0 < c.n_term; t0 += 5) {
+            double vals[16];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                vals[3 * j] = vals[3 * j + 1] = vals[3 * j + 2] = 0.0;
+                if (t0 + j >= c.n_term) continue;
+                const int l = c.term_l[t0 + j], f = c.term_f[t0 + j];
+                double2 yc = c0, yq = q0;
+                if (f >= 0) {
+                    const int *so = S.f_sl_off + (size_t)f * (S.n_slices + 1);
+                    const int off = so[sl] + lane, width = (so[sl + 1] - so[sl]) / kSlice;
+                    yc = yq = zero;
+                    for (int k = 0; k < width; ++k) {
+                        const double gv = S.f_val[off + k * kSlice];
+                        const int col = S.f_cols[off + k * kSlice];
+                        const double2 a1 = m.C[col], a2 = Q[col];
+                        yc.x = fma(gv, a1.x, yc.x); yc.y = fma(gv, a1.y, yc.y);
+                        yq.x = fma(gv, a2.x, yq.x); yq.y = fma(gv, a2.y, yq.y);
+                    }
+                }
+                const double v = c.v[l], dv = c.dv[l];
+                w.x = fma(v, yc.x, w.x); w.y = fma(v, yc.y, w.y);
+                u.x = fma(dv, yc.x, u.x); u.y = fma(dv, yc.y, u.y);
+                mq.x = fma(v, yq.x, mq.x); mq.y = fma(v, yq.y, mq.y);
+                vals[3 * j] = z0.x * yc.y - z0.y * yc.x;
+                vals[3 * j + 1] = -(c0.x * yc.x + c0.y * yc.y);
+                vals[3 * j + 2] = -(d0.x * yc.x + d0.y * yc.y);
+            }
+            vals[15] = t0 == 0 ? z0.x * d0.x + z0.y * d0.y : 0.0;
+            const double x = reduce16(vals, lane);
+            const int i = lane >> 1;
+            if (!(lane & 1)) {
+                if (i == 15) wt[1] += x;
+                else if (t0 + i / 3 < c.n_term) wt[4 + 3 * c.term_l[t0 + i / 3] + i % 3] += x;
+            }
+            __syncwarp();
+        }
+        if (in) {
+            m.W[r] = w;
+            m.U[r] = u;
+            m.MDC[r] = mq;
+        }
+    }
+    __syncthreads();
+    const double h = c.hp;
+    for (int r = tid; r < n; r += nt) {
+        const int ru = S.up[r], rd = S.dn[r];
+        const double au = S.aup[r], ad = S.adn[r];
+        const double2 kbu = m.KB[ru], kbd = m.KB[rd], wu = m.W[ru], wd = m.W[rd], u = m.U[r], mq = m.MDC[r];
+        const double2 Dkb = make_double2(ad * kbd.x - au * kbu.x, ad * kbd.y - au * kbu.y);
+        const double2 Dw = make_double2(ad * wd.x - au * wu.x, ad * wd.y - au * wu.y);
+        // abar_in = conj(p) (i M z - PPhibar M D c - 2 PRbar u + PPhibar D w) - h D kbar
+        const double2 x = cconjmul<double>(m.PH[S.lev[r]], make_double2(fma(PPb, Dw.x, fma(-2.0 * PRb, u.x, mq.x)),
+                                                                        fma(PPb, Dw.y, fma(-2.0 * PRb, u.y, mq.y))));
+        double2 o = m.YN[r];
+        o.x += fma(-h, Dkb.x, x.x);
+        o.y += fma(-h, Dkb.y, x.y);
+        m.YN[r] = o;
+    }
+    cross_warp(4 + 3 * L, c, wred);
+    if (warp == 0) {
+        // s1 = Re(kbar^dag (-i conj(p) M' c)), s2 = Re(kbar^dag D a), s3 = Re(c^dag M'' c), s4 = -Re((Dc)^dag M' c)
+        double S1 = 0.0, S3 = 0.0, S4 = 0.0;
+        for (int l = lane; l < L; l += 32) {
+            S1 = fma(c.dv[l], c.red[4 + 3 * l], S1);
+            S3 = fma(-c.d2v[l], c.red[5 + 3 * l], S3);
+            S4 = fma(c.dv[l], c.red[6 + 3 * l], S4);
+        }
+        S1 = wsum(S1); S3 = wsum(S3); S4 = wsum(S4);
+        const double S2 = c.red[1], Rb = c.kb[0], Phb = c.kb[2], ir = 1.0 / R_, imu = 1.0 / mu;
+        const double ir2 = ir * ir, ir3 = ir2 * ir, g = PP * ir3 * imu;
+        if (lane == 0) {
+            c.ynew[0] += S1 - g * S2 + PRb * (-S3 - 3.0 * g * PP * ir) - 2.0 * g * Phb + PPb * S4;
+            c.ynew[1] += Rb * imu;
+            c.ynew[3] += 0.5 * S2 * ir2 * imu + PRb * 2.0 * g + Phb * ir2 * imu;
+        }
+    }
+    // parameters: sum_l dv_lp (alpha_l + PPhibar gamma_l) + d(dv)_lp PRbar beta_l, one parameter per warp, one
+    // term per lane
+    {
+        const int k = c.kint;
+        const double x = c.x;
+        for (int pp = warp; pp < S.P; pp += nw) {
+            double acc = 0.0;
+            for (int l = lane; l < L; l += 32) {
+                const dbl4 q = S.dvcoef[((size_t)pp * L + l) * S.n_int + k];
+                const double dvl = q.x + x * (q.y + x * (q.z + x * q.w));
+                const double ddvl = q.y + x * (2.0 * q.z + 3.0 * x * q.w);
+                acc += dvl * fma(PPb, c.red[6 + 3 * l], c.red[4 + 3 * l]) + ddvl * (PRb * c.red[5 + 3 * l]);
+            }
+            acc = wsum(acc);
+            if (lane == 0) c.theta[pp] += acc;
+        }
+    }
+    __syncthreads();
+}
+
+// The same in the mixed precision (FP32 vectors).
+__device__ void vjp_eval32(const DevSys &S, double t, unsigned n_half, const float2 *Ya, const double *Yq,
+                         AdjSmem<float> &m, AdjCtl<float> &c, float *wred)
+{
+    using R = float;
     using V = typename Cx<R>::T;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const int n = S.n, L = S.L;
@@ -308,8 +474,7 @@ __device__ void vjp_eval(const DevSys &S, double t, unsigned n_half, const typen
     __syncthreads();
     for (int r = tid; r < n; r += nt) {
         R au, ad;
-        if constexpr (sizeof(R) == 8) { au = S.aup[r]; ad = S.adn[r]; }
-        else { au = S.aupf[r]; ad = S.adnf[r]; }
+        au = S.aupf[r]; ad = S.adnf[r];
         const V cu = m.C[S.up[r]], cd = m.C[S.dn[r]];
         m.DC[r] = Cx<R>::mk(ad * cd.x - au * cu.x, ad * cd.y - au * cu.y);
     }
@@ -349,9 +514,7 @@ __device__ void vjp_eval(const DevSys &S, double t, unsigned n_half, const typen
             V yc = Cx<R>::mk(0, 0), yz = yc, yd = yc;
             for (int k = 0; k < width; ++k) {
                 const int e = off + k * kSlice + lane;
-                R gv;
-                if constexpr (sizeof(R) == 8) gv = S.f_val[e];
-                else gv = S.f_valf[e];
+                const R gv = S.f_valf[e];
                 const int col = S.f_cols[e];
                 const V a1 = m.C[col], a2 = m.Z[col], a3 = m.DC[col];
                 yc.x = fma(gv, a1.x, yc.x); yc.y = fma(gv, a1.y, yc.y);
@@ -383,8 +546,7 @@ __device__ void vjp_eval(const DevSys &S, double t, unsigned n_half, const typen
     for (int r = tid; r < n; r += nt) {
         const int ru = S.up[r], rd = S.dn[r];
         R au, ad;
-        if constexpr (sizeof(R) == 8) { au = S.aup[r]; ad = S.adn[r]; }
-        else { au = S.aupf[r]; ad = S.adnf[r]; }
+        au = S.aupf[r]; ad = S.adnf[r];
         const V p = m.PH[S.lev[r]], kb = m.KB[r];
         const V kbu = m.KB[ru], kbd = m.KB[rd];
         const V wu = m.W[ru], wd = m.W[rd];
@@ -439,18 +601,11 @@ __device__ void vjp_eval(const DevSys &S, double t, unsigned n_half, const typen
         for (int pp = warp; pp < S.P; pp += nw) {
             R acc = 0;
             for (int l = lane; l < L; l += 32) {
-                if constexpr (sizeof(R) == 8) {
-                    const dbl4 q = S.dvcoef[((size_t)pp * L + l) * S.n_int + k];
-                    const double dvl = q.x + x * (q.y + x * (q.z + x * q.w));
-                    const double ddvl = q.y + x * (2.0 * q.z + 3.0 * x * q.w);
-                    acc += dvl * c.ab[0][l] + ddvl * c.ab[1][l];
-                } else {
-                    const float4 q = S.dvcoef_f[((size_t)pp * L + l) * S.n_int + k];
-                    const float xf = (float)x;
-                    const float dvl = fmaf(xf, fmaf(xf, fmaf(xf, q.w, q.z), q.y), q.x);
-                    const float ddvl = fmaf(xf, fmaf(3.0f * xf, q.w, 2.0f * q.z), q.y);
-                    acc += dvl * c.ab[0][l] + ddvl * c.ab[1][l];
-                }
+                const float4 q = S.dvcoef_f[((size_t)pp * L + l) * S.n_int + k];
+                const float xf = (float)x;
+                const float dvl = fmaf(xf, fmaf(xf, fmaf(xf, q.w, q.z), q.y), q.x);
+                const float ddvl = fmaf(xf, fmaf(3.0f * xf, q.w, 2.0f * q.z), q.y);
+                acc += dvl * c.ab[0][l] + ddvl * c.ab[1][l];
             }
             acc = wsum(acc);
             if (lane == 0) c.theta[pp] += (double)acc;
@@ -459,8 +614,11 @@ __device__ void vjp_eval(const DevSys &S, double t, unsigned n_half, const typen
     __syncthreads();
 }
 
+// two CTAs per SM in the mixed precision, whose barriers and chains then fill each other's gaps (its FP64
+// counterpart fills the FP64 pipe and its shared memory with one): N = 441, 256 trajectories 498 -> 313 ms together
+// with the kept stage states
 template <class R>
-__global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjArgs a)
+__global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 2 : 1) k_adjoint(AdjArgs a)
 {
     using V = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -468,7 +626,13 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjArgs a)
     __shared__ DevSys S;
     __shared__ R wred[kAdjWarps * kAdjRed];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) S = *a.sys;
+    if (tid == 0) {
+        S = *a.sys;
+        c.n_term = 0;
+        for (int l = 0; l < S.L; ++l)
+            if ((S.id_mask >> l) & 1ull) { c.term_l[c.n_term] = l; c.term_f[c.n_term++] = -1; }
+        for (int f = 0; f < S.n_f; ++f) { c.term_l[c.n_term] = S.f_term[f]; c.term_f[c.n_term++] = f; }
+    }
     __syncthreads();
     const int n = S.n;
     AdjSmem<R> m;
@@ -478,7 +642,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjArgs a)
     m.A = base; m.E = m.A + n; m.Y2 = m.E + n; m.Y3 = m.Y2 + n; m.Y4 = m.Y3 + n; m.K = m.Y4 + n; m.ACC = m.K + n;
     m.C = m.ACC + n; m.W = m.C + n; m.LAM = m.W + n; m.KB = m.LAM + n; m.YN = m.KB + n; m.Z = m.YN + n;
     m.DC = m.Z + n; m.MZ = m.DC + n; m.MDC = m.MZ + n; m.U = m.MDC + n; m.PH = m.U + n;
-    unsigned char *scr = a.scratch + (size_t)blockIdx.x * (size_t)(a.max_ckpt + a.K) * a.stride;
+    unsigned char *scr = a.scratch + (size_t)blockIdx.x * ((size_t)a.max_ckpt * a.stride + (size_t)a.K * a.seg_stride);
     unsigned char *ck = scr, *seg = scr + (size_t)a.max_ckpt * a.stride;
     const double cst[4] = {0.0, 0.5, 0.5, 1.0};
     const unsigned hst[4] = {0u, 1u, 1u, 2u};
@@ -616,16 +780,30 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjArgs a)
                 load_state(ck + (size_t)sg * a.stride, c.q);
                 __syncthreads();
                 for (int st = n0; st < n1; ++st) {
-                    store_state(seg + (size_t)(st - n0) * a.stride, c.q);
+                    unsigned char *rec = seg + (size_t)(st - n0) * a.seg_stride;
+                    store_state(rec, c.q);
                     __syncthreads();
-                    if (st + 1 < n1) fwd_step(st);
+                    if (st + 1 < n1 || a.stages) fwd_step(st);
+                    if (a.stages) {
+                        V *y = reinterpret_cast<V *>(rec + a.stride);
+                        for (int r = tid; r < n; r += nt) { y[r] = m.Y2[r]; y[n + r] = m.Y3[r]; y[2 * n + r] = m.Y4[r]; }
+                        if (tid < 16) reinterpret_cast<double *>(rec + a.seg_stride)[tid - 16] = c.qk[tid >> 2][tid & 3];
+                        __syncthreads();
+                    }
                 }
                 for (int st = n1 - 1; st >= n0; --st) {
                     // stage states of step st
-                    load_state(seg + (size_t)(st - n0) * a.stride, c.q);
-                    __syncthreads();
-                    fwd_step(st);  // leaves Y2..Y4 and c.qk; A now holds y_{st+1} (unused)
-                    load_state(seg + (size_t)(st - n0) * a.stride, c.q);
+                    const unsigned char *rec = seg + (size_t)(st - n0) * a.seg_stride;
+                    if (a.stages) {
+                        const V *y = reinterpret_cast<const V *>(rec + a.stride);
+                        for (int r = tid; r < n; r += nt) { m.Y2[r] = y[r]; m.Y3[r] = y[n + r]; m.Y4[r] = y[2 * n + r]; }
+                        if (tid < 16) c.qk[tid >> 2][tid & 3] = reinterpret_cast<const double *>(rec + a.seg_stride)[tid - 16];
+                    } else {
+                        load_state(rec, c.q);
+                        __syncthreads();
+                        fwd_step(st);  // leaves Y2..Y4 and c.qk; A now holds y_{st+1} (unused)
+                    }
+                    load_state(rec, c.q);
                     __syncthreads();
                     // ynew = lam; kbar4 = dt/6 lam
                     const R h6 = (R)(dt / 6.0);
@@ -647,7 +825,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjArgs a)
                         // keep ynew before this stage (K is free here) to form Ybar_s = after - before
                         for (int r = tid; r < n; r += nt) m.K[r] = m.YN[r];
                         __syncthreads();
-                        vjp_eval<R>(S, t0 + cst[s] * dt, 2u * st + hst[s], Ya, c.qk[s], m, c, wred);
+                        if constexpr (fp32) vjp_eval32(S, t0 + cst[s] * dt, 2u * st + hst[s], Ya, c.qk[s], m, c, wred);
+                        else vjp_eval64(S, t0 + cst[s] * dt, Ya, c.qk[s], m, c, wred);
                         if (s > 0) {
                             // Ybar_s = YN - K(before); next kbar = wprev * lam + bprev * Ybar_s
                             const double wl = (s == 1) ? dt / 6.0 : dt / 3.0;
@@ -774,6 +953,10 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     const size_t rsz = fp32 ? sizeof(float) : sizeof(double);
     const size_t amp_bytes = ((fp32 ? 4 : 2) * (size_t)h.n * rsz + 15) & ~(size_t)15;
     const size_t stride = amp_bytes + 32;
+    // a recomputed step keeps its three later stage states and the classical stage states too: the reverse
+    // sweep then needs no second recomputation (a fifth of a gradient); left out when the segments of all
+    // CTAs would take more than 16 GB
+    const size_t stage_bytes = ((6 * (size_t)h.n * rsz + 15) & ~(size_t)15) + 16 * sizeof(double);
     // work vectors: 17 of length N and the phase factors of every level, in shared memory when
     // they fit, else in a global-memory region per CTA
     const size_t vsz = fp32 ? sizeof(float2) : sizeof(double2);
@@ -793,6 +976,8 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, smem)) != cudaSuccess)
         return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     const int grid = std::max(1, std::min(n, sms * std::max(per_sm, 1)));
+    const bool stages = (size_t)grid * ckpt * (stride + stage_bytes) <= (size_t)16 << 30;
+    const size_t seg_stride = stride + (stages ? stage_bytes : 0);
     std::vector<void *> tmp;
     auto get = [&](void **p, size_t b) {
         cudaError_t r = cudaMallocAsync(p, b ? b : 16, st);
@@ -824,12 +1009,13 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     }
     aa.dLds = (const double *)ptr;
     aa.n = n; aa.n_groups = n_groups; aa.K = ckpt; aa.max_ckpt = max_ckpt; aa.stride = stride;
+    aa.seg_stride = seg_stride; aa.stages = stages ? 1 : 0;
     int *queue = nullptr;
     unsigned char *scratch = nullptr, *vec = nullptr;
     double *theta = nullptr, *out = nullptr;
     int *status = nullptr;
     if ((e = get((void **)&queue, sizeof(int))) != cudaSuccess ||
-        (e = get((void **)&scratch, (size_t)grid * (max_ckpt + ckpt) * stride)) != cudaSuccess ||
+        (e = get((void **)&scratch, (size_t)grid * ((size_t)max_ckpt * stride + (size_t)ckpt * seg_stride))) != cudaSuccess ||
         (vec_global && (e = get((void **)&vec, (size_t)grid * vec_bytes)) != cudaSuccess) ||
         (e = get((void **)&theta, sizeof(double) * (size_t)n * h.P)) != cudaSuccess ||
         (e = get((void **)&status, sizeof(int) * (size_t)n)) != cudaSuccess ||
