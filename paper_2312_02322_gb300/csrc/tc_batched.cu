@@ -40,6 +40,17 @@ constexpr long long kTcWait = 1ll << 24;
 
 enum { TS_IDLE = 0, TS_ACTIVE = 1, TS_FINAL = 2, TS_WAIT = 3 };
 
+// packed FP32 fused multiply-add, each half rounded as the scalar instruction
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+          "l"(reinterpret_cast<const unsigned long long &>(c)));
+    return d;
+}
+
 // per-slot values that are not per component (the four component lanes of a slot read them)
 struct TSlot {
     double dt, h6, r_end, e0, j0, ndev, edev, jdev;
@@ -80,33 +91,6 @@ __device__ __forceinline__ uint16_t bf16_rn(float x) { return __bfloat16_as_usho
 __device__ __forceinline__ float bf16_f(uint16_t h) { return __bfloat162float(__ushort_as_bfloat16(h)); }
 
 // ---------------------------------------------------------------------------------------------
-// the inputs of one element update (row r, slot sl) gathered from global memory
-struct ElemIn {
-    float2 c, cu, cd, p, q, a0, acc;
-    float au, ad;
-    int lev;
-};
-
-// gather: only loads, so that several elements' loads are in flight before any store
-__device__ __forceinline__ void tc_elem_gather(const TcState &T, const DevSys &S, int s, int cur, int r, int sl,
-                                               ElemIn &in)
-{
-    const size_t e = (size_t)r * T.S + sl;
-    const float2 *Cc = T.C[cur];
-    const float2 *PHc = (s == 0 || s == 3) ? T.PHa : T.PHb;
-    const float2 *PHn = (s == 0 || s == 1) ? T.PHb : T.PHa;
-    in.c = __ldg(Cc + e);
-    in.au = __ldg(S.aupf + r);
-    in.ad = __ldg(S.adnf + r);
-    in.cu = __ldg(Cc + (size_t)__ldg(S.up + r) * T.S + sl);
-    in.cd = __ldg(Cc + (size_t)__ldg(S.dn + r) * T.S + sl);
-    in.lev = __ldg(S.lev + r);
-    in.p = __ldg(PHc + (size_t)in.lev * T.S + sl);
-    in.q = __ldg(PHn + (size_t)in.lev * T.S + sl);
-    in.a0 = T.A[e];
-    in.acc = T.ACC[e];
-}
-
 // the update of one element from w = M c and u = M' c (Eq. 5, RK4) and its inputs; adds its force,
 // torque and (stage 0) diagnostic contributions to part[6] (FP32: a thread sums a few rows; the
 // sums across threads, row tiles and the classical update are FP64 -- the FP64 pipe of this GPU is
@@ -189,41 +173,43 @@ __device__ __forceinline__ void elem_store(const TcState &T, const DevSys &S, in
     }
 }
 
-__device__ __forceinline__ void tc_elem_apply(const TcState &T, const DevSys &S, int s, int cur, int r, int sl,
-                                              int st, const ElemIn &in, float2 w, float2 u, float *part)
-{
-    if (st == TS_IDLE) return;
-    const bool is_s0 = st == TS_WAIT && s == 3 && r == T.slot[sl].s0;
-    const float elev = (st == TS_ACTIVE || st == TS_FINAL) && s == 0 ? S.lev_energy_f[in.lev] : 0.f;
-    float2 a, acc, c;
-    const int mode = elem_core(s, st, is_s0, in.c, in.cu, in.cd, in.p, in.q, in.a0, in.acc, in.au, in.ad, elev,
-                               T.hp[sl], T.dtf[sl], w, u, part, a, acc, c);
-    elem_store(T, S, cur, r, sl, mode, a, acc, c);
-}
-
 // ---------------------------------------------------------------------------------------------
 // one RK4 stage of every element: one CTA per (row tile, 64-slot tile).
-//  - B operand: the tile's phase-rotated amplitudes as BF16 hi/lo, built once;
-//  - the G^l tiles (BF16 hi/lo) stream through a two-deep shared-memory ring by bulk TMA copies
-//    (warp 17); warp 16 issues, per term, the MMAs of the non-zero K chunks (three per chunk:
-//    hi.hi + hi.lo + lo.hi) into one of two TMEM accumulators, Y_l = G^l C;
-//  - sixteen epilogue warps (four per TMEM lane quadrant, 32 columns each) fold each term into
-//    w += v_l Y_l and u += v_l' Y_l with the per-slot spline weights (Eq. 12), in registers;
-//  - the element update of Eq. 5 and RK4 (tc_elem_gather / tc_elem_apply, four rows' loads in
-//    flight per thread) runs on the staged w, u with the identity
-//    terms added, and the per-slot partial sums of force, torque and diagnostics over the
-//    tile's rows go to part[row tile][slot].
+//  - the products are formed transposed, Y_l^T = C^T (G^l)^T: the A operand is the tile's phase-rotated amplitudes
+//    (128 real columns = Re, Im of the slots; K = the tile's rows) as BF16 hi/lo, written to tensor memory
+//    once per stage; the B operand is the G^l tile (BF16 hi/lo, symmetric), streamed through a three-deep
+//    shared-memory ring by bulk TMA copies (warp 17).  An MMA then reads one operand from shared
+//    memory instead of two;
+//  - warp 16 issues, per term, the MMAs of the non-zero K chunks (three per chunk: hi.hi + lo.hi + hi.lo) into
+//    one of two TMEM accumulators (lane = real column, column = row);
+//  - sixteen epilogue warps (four per TMEM lane quadrant, 32 rows each) fold each term into
+//    w += v_l Y_l and u += v_l' Y_l (Eq. 12) with the weights of the lane's slot, in registers;
+//  - the element update of Eq. 5 and RK4 (four rows' loads in flight per thread) runs on the staged w, u with
+//    the identity terms added; per-row quantities wait in shared memory, so that no load of it depends on
+//    another; the per-slot partial sums of force, torque and diagnostics over the tile's rows go to
+//    part[row tile][slot].
+// N = 1580 (27 terms, 532 MMAs of 128 x 128 x 16 per CTA), cycles per CTA: operand 6.7 -> 7.4 k, products 64 -> 54 k
+// (75 per MMA against 118 with both operands in shared memory and descriptors formed per MMA; the tensor pipe's own
+// 67), update 25 -> 14 k (per-row indices from shared memory).  The products bound it.
 constexpr int kTcEpiWarps = 16;
 constexpr int kTcMmaWarp = kTcEpiWarps, kTcLoadWarp = kTcEpiWarps + 1;
 constexpr int kTcThreads = 32 * (kTcEpiWarps + 2);
-constexpr uint32_t kTcTileBytes = 2u * 128u * 128u * 2u;  // a G tile or the B operand, hi + lo
-constexpr size_t kTcSmemFixed = 3 * (size_t)kTcTileBytes;  // A ring (2) + B operand
+constexpr int kTcRing = 3;
+constexpr uint32_t kTcTileBytes = 2u * 128u * 128u * 2u;  // a G tile, hi + lo
+constexpr size_t kTcSmemFixed = kTcRing * (size_t)kTcTileBytes;
 constexpr int kTcWs = kTcSlotsPerTile + 1;                  // padded row of the staged w, u
+constexpr uint32_t kTcColA = 256;                           // TMEM columns: two accumulators, then C^T hi, lo (64 each)
+
+// what the element update needs of a row
+struct RowInfo {
+    int up, dn, lev;
+    float au, ad, elev;
+};
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, int cur)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
-    __shared__ __align__(8) uint64_t bar_full[2], bar_mma[2], bar_epi[2], bar_drain;
+    __shared__ __align__(8) uint64_t bar_full[kTcRing], bar_ring[kTcRing], bar_mma[2], bar_epi[2], bar_drain;
     __shared__ uint32_t tmem_base;
     __shared__ int any_live, err;
     const DevSys &S = *T.sys;
@@ -240,82 +226,96 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, in
     }
     __syncthreads();
     if (!any_live) return;
-    unsigned char *Aring = sm, *Bop = sm + 2 * kTcTileBytes;
+    unsigned char *ring = sm;
     float *s_v = reinterpret_cast<float *>(sm + kTcSmemFixed), *s_dv = s_v + nf * kTcSlotsPerTile;
     const float2 *Cg = T.C[cur];
-    // per-term spline weights of the tile's slots
-    for (int i = tid; i < nf * kTcSlotsPerTile; i += kTcThreads) {
-        const int f = i / kTcSlotsPerTile, j = i % kTcSlotsPerTile, l = S.f_term[f];
-        s_v[i] = T.coef[(size_t)l * T.S + s0 + j];
-        s_dv[i] = T.coef[((size_t)S.L + l) * T.S + s0 + j];
-    }
-    // B operand: real column n = 2j + (Re, Im) of slot j, K = row k of the tile; 8 rows of one
-    // slot per task, written as 16-byte core-matrix rows
-    for (int task = tid; task < kTcSlotsPerTile * 16; task += kTcThreads) {
-        const int j = task % kTcSlotsPerTile, o = task / kTcSlotsPerTile;
-        uint32_t rh[4], rl[4], ih[4], il[4];
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-            float2 c0 = make_float2(0.f, 0.f), c1 = make_float2(0.f, 0.f);
-            const int k = 8 * o + i;
-            if (k < R) c0 = Cg[(size_t)(r0 + k) * T.S + s0 + j];
-            if (k + 1 < R) c1 = Cg[(size_t)(r0 + k + 1) * T.S + s0 + j];
-            const uint16_t h0 = bf16_rn(c0.x), h1 = bf16_rn(c1.x), g0 = bf16_rn(c0.y), g1 = bf16_rn(c1.y);
-            rh[i / 2] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-            ih[i / 2] = (uint32_t)g0 | ((uint32_t)g1 << 16);
-            rl[i / 2] = (uint32_t)bf16_rn(c0.x - bf16_f(h0)) | ((uint32_t)bf16_rn(c1.x - bf16_f(h1)) << 16);
-            il[i / 2] = (uint32_t)bf16_rn(c0.y - bf16_f(g0)) | ((uint32_t)bf16_rn(c1.y - bf16_f(g1)) << 16);
-        }
-        const uint32_t ore = tc_kmajor_offset(2 * j, 8 * o, 16), oim = tc_kmajor_offset(2 * j + 1, 8 * o, 16);
-        *reinterpret_cast<uint4 *>(Bop + ore) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
-        *reinterpret_cast<uint4 *>(Bop + kTcTileBytes / 2 + ore) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
-        *reinterpret_cast<uint4 *>(Bop + oim) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
-        *reinterpret_cast<uint4 *>(Bop + kTcTileBytes / 2 + oim) = make_uint4(il[0], il[1], il[2], il[3]);
-    }
     if (warp == kTcMmaWarp) {
-        tc_tmem_alloc(&tmem_base, 256);
+        tc_tmem_alloc(&tmem_base, 512);
         tc_tmem_relinquish();
     }
     if (tid == 0) {
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kTcRing; ++b) {
             tc_mbar_init(&bar_full[b], 1);
+            tc_mbar_init(&bar_ring[b], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
             tc_mbar_init(&bar_mma[b], 1);
             tc_mbar_init(&bar_epi[b], kTcEpiWarps);
         }
         tc_mbar_init(&bar_drain, 1);
     }
-    tc_fence_proxy_async();
+    // per-term spline weights of the tile's slots, per-row quantities
+    for (int i = tid; i < nf * kTcSlotsPerTile; i += kTcThreads) {
+        const int f = i / kTcSlotsPerTile, j = i % kTcSlotsPerTile, l = S.f_term[f];
+        s_v[i] = T.coef[(size_t)l * T.S + s0 + j];
+        s_dv[i] = T.coef[((size_t)S.L + l) * T.S + s0 + j];
+    }
+    RowInfo own{};
+    if (tid < R) {
+        const int r = r0 + tid, lev = S.lev[r];
+        own = RowInfo{S.up[r], S.dn[r], lev, S.aupf[r], S.adnf[r], S.lev_energy_f[lev]};
+    }
+    tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tbase = tmem_base;
-    float w[32], u[32];
+    if (warp < kTcEpiWarps) {
+        // A operand: lane m = 2 j + (Re, Im) of slot j, 32 of the K = 128 rows per warp, two BF16 per column
+        const int q = warp & 3, kq = warp >> 2;
+        const float *src = reinterpret_cast<const float *>(Cg + (size_t)(r0 + 32 * kq) * T.S + s0) + 32 * q + lane;
+        uint32_t hi[16], lo[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k = 32 * kq + 2 * i;
+            const float x0 = k < R ? __ldg(src + (size_t)(2 * i) * 2 * T.S) : 0.f;
+            const float x1 = k + 1 < R ? __ldg(src + (size_t)(2 * i + 1) * 2 * T.S) : 0.f;
+            const uint16_t h0 = bf16_rn(x0), h1 = bf16_rn(x1);
+            hi[i] = (uint32_t)h0 | ((uint32_t)h1 << 16);
+            lo[i] = (uint32_t)bf16_rn(x0 - bf16_f(h0)) | ((uint32_t)bf16_rn(x1 - bf16_f(h1)) << 16);
+        }
+        const uint32_t ta = tbase + ((uint32_t)(32 * q) << 16) + kTcColA + 16 * kq;
+        tc_st16(ta, hi);
+        tc_st16(ta + 64, lo);
+        tc_wait_st();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    float2 w[16], u[16];  // pairs of rows
     if (warp == kTcLoadWarp) {
-        // ---- bulk copies of the G tiles into the ring (lane 0); slot f & 1 is free once the
-        // MMAs of term f - 2 completed
+        // ---- bulk copies of the G tiles into the ring (lane 0); a buffer is free once the MMAs of the
+        // term it held before completed
         if (lane == 0) {
             const unsigned char *gt = reinterpret_cast<const unsigned char *>(S.g_tiles);
             int f = 0;
             for (; f < nf; ++f) {
-                const int b = f & 1;
-                if (f >= 2 && !tc_mbar_wait(&bar_mma[b], ((f - 2) >> 1) & 1, kTcWait)) {
+                const int b = f % kTcRing;
+                if (f >= kTcRing && !tc_mbar_wait(&bar_ring[b], (f / kTcRing - 1) & 1, kTcWait)) {
                     err = 1;
                     break;
                 }
                 tc_mbar_expect_tx(&bar_full[b], kTcTileBytes);
-                tc_bulk_g2s(Aring + b * kTcTileBytes, gt + ((size_t)f * nt + rt) * kTcTileBytes, kTcTileBytes,
+                tc_bulk_g2s(ring + b * kTcTileBytes, gt + ((size_t)f * nt + rt) * kTcTileBytes, kTcTileBytes,
                             &bar_full[b]);
             }
             // before the buffers are released: the last copies issued have landed
-            for (int k = f - 1; k >= 0 && k >= f - 2; --k) tc_mbar_wait(&bar_full[k & 1], (k >> 1) & 1, kTcWait);
+            for (int k = f - 1; k >= 0 && k >= f - kTcRing; --k)
+                tc_mbar_wait(&bar_full[k % kTcRing], (k / kTcRing) & 1, kTcWait);
         }
     } else if (warp == kTcMmaWarp) {
-        // ---- MMA issue (lane 0)
+        // ---- MMA issue (one lane).  The descriptors of the three ring buffers are formed once and advance by
+        // 256 bytes (16 in the address field) per K chunk: a single thread issues every MMA, so the
+        // instructions between two of them are what the tensor pipe would wait for
         if (lane == 0) {
             const uint32_t idesc = tc_idesc_bf16_f32(128, 128);
-            const uint32_t b_hi = tc_smem_addr(Bop), b_lo = b_hi + kTcTileBytes / 2;
-            for (int f = 0; f < nf; ++f) {
+            const uint32_t a_hi = tbase + kTcColA, a_lo = a_hi + 64;
+            const uint64_t g0 = tc_sdesc(tc_smem_addr(ring), 128, 2048);
+            const uint8_t *kmp = S.g_kmask + rt;
+            uint32_t km = nf > 0 ? __ldg(kmp) : 0u;
+            for (int f = 0, rb = 0; f < nf; ++f) {
                 const int b = f & 1;
-                bool ok = tc_mbar_wait(&bar_full[b], (f >> 1) & 1, kTcWait);
+                const uint32_t km_next = f + 1 < nf ? __ldg(kmp + (size_t)(f + 1) * nt) : 0u;
+                bool ok = tc_mbar_wait(&bar_full[rb], (f / kTcRing) & 1, kTcWait);
                 if (ok && f >= 2) ok = tc_mbar_wait(&bar_epi[b], ((f - 2) >> 1) & 1, kTcWait);
                 if (!ok) {
                     // the MMAs already issued complete before the accumulators are released
@@ -325,50 +325,46 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, in
                     break;
                 }
                 tc_fence_after_sync();
-                const uint32_t a_hi = tc_smem_addr(Aring + b * kTcTileBytes), a_lo = a_hi + kTcTileBytes / 2;
+                const uint64_t g_hi = g0 + (uint64_t)(rb * (kTcTileBytes >> 4)), g_lo = g_hi + (kTcTileBytes >> 5);
                 const uint32_t d = tbase + 128u * b;
-                const uint32_t km = S.g_kmask[(size_t)f * nt + rt];
                 bool acc = false;
+#pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     if (!((km >> ks) & 1u)) continue;
-                    const uint32_t o = ks * 256;
-                    tc_mma_bf16(d, tc_sdesc(a_hi + o, 128, 2048), tc_sdesc(b_hi + o, 128, 2048), idesc, acc);
-                    tc_mma_bf16(d, tc_sdesc(a_hi + o, 128, 2048), tc_sdesc(b_lo + o, 128, 2048), idesc, true);
-                    tc_mma_bf16(d, tc_sdesc(a_lo + o, 128, 2048), tc_sdesc(b_hi + o, 128, 2048), idesc, true);
+                    tc_mma_bf16_ta(d, a_hi + 8 * ks, g_hi + 16 * ks, idesc, acc);
+                    tc_mma_bf16_ta(d, a_lo + 8 * ks, g_hi + 16 * ks, idesc, true);
+                    tc_mma_bf16_ta(d, a_hi + 8 * ks, g_lo + 16 * ks, idesc, true);
                     acc = true;
                 }
                 tc_commit(&bar_mma[b]);
+                tc_commit(&bar_ring[rb]);
+                km = km_next;
+                rb = rb + 1 < kTcRing ? rb + 1 : 0;
             }
         }
     } else {
-        // ---- epilogue warps: lanes of quadrant warp % 4, columns 32 * (warp / 4) .. + 31
-        const int q = warp & 3, hcol = 32 * (warp >> 2);
+        // ---- epilogue warps: lanes of quadrant warp % 4, rows 32 * (warp / 4) .. + 31
+        const int q = warp & 3, hrow = 32 * (warp >> 2), j = 16 * q + (lane >> 1);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) { w[i] = 0.f; u[i] = 0.f; }
+        for (int i = 0; i < 16; ++i) w[i] = u[i] = make_float2(0.f, 0.f);
         for (int f = 0; f < nf; ++f) {
             const int b = f & 1;
+            const float v = s_v[f * kTcSlotsPerTile + j], dv = s_dv[f * kTcSlotsPerTile + j];
             if (!tc_mbar_wait(&bar_mma[b], (f >> 1) & 1, kTcWait)) { err = 1; break; }
+            __syncwarp();
             tc_fence_after_sync();
-            const float *vf = s_v + f * kTcSlotsPerTile + hcol / 2, *dvf = s_dv + f * kTcSlotsPerTile + hcol / 2;
-            const uint32_t ta = tbase + 128u * b + ((uint32_t)(32 * q) << 16) + hcol;
+            const uint32_t ta = tbase + 128u * b + ((uint32_t)(32 * q) << 16) + hrow;
+            const float2 v2 = make_float2(v, v), dv2 = make_float2(dv, dv);
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
                 uint32_t d[16];
                 tc_ld16_raw(ta + 16 * hh, d);
                 tc_wait_ld_16(d);
 #pragma unroll
-                for (int c = 0; c < 16; c += 4) {
-                    const float2 v2 = *reinterpret_cast<const float2 *>(vf + 8 * hh + (c >> 1));
-                    const float2 dv2 = *reinterpret_cast<const float2 *>(dvf + 8 * hh + (c >> 1));
-                    const int o = 16 * hh + c;
-                    w[o] = fmaf(v2.x, __uint_as_float(d[c]), w[o]);
-                    w[o + 1] = fmaf(v2.x, __uint_as_float(d[c + 1]), w[o + 1]);
-                    w[o + 2] = fmaf(v2.y, __uint_as_float(d[c + 2]), w[o + 2]);
-                    w[o + 3] = fmaf(v2.y, __uint_as_float(d[c + 3]), w[o + 3]);
-                    u[o] = fmaf(dv2.x, __uint_as_float(d[c]), u[o]);
-                    u[o + 1] = fmaf(dv2.x, __uint_as_float(d[c + 1]), u[o + 1]);
-                    u[o + 2] = fmaf(dv2.y, __uint_as_float(d[c + 2]), u[o + 2]);
-                    u[o + 3] = fmaf(dv2.y, __uint_as_float(d[c + 3]), u[o + 3]);
+                for (int i = 0; i < 8; ++i) {
+                    const float2 y = make_float2(__uint_as_float(d[2 * i]), __uint_as_float(d[2 * i + 1]));
+                    w[8 * hh + i] = fma2(v2, y, w[8 * hh + i]);
+                    u[8 * hh + i] = fma2(dv2, y, u[8 * hh + i]);
                 }
             }
             tc_fence_before_sync();
@@ -376,46 +372,66 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, in
             if (lane == 0) tc_mbar_arrive(&bar_epi[b]);
         }
     }
+    __syncwarp();
     __syncthreads();
-    // stage w and u through shared memory (the ring and B buffers are free now)
+    // stage w and u through shared memory (the ring is free now)
     float2 *Wst = reinterpret_cast<float2 *>(sm), *Ust = Wst + 128 * kTcWs;
     float *red = reinterpret_cast<float *>(Ust + 128 * kTcWs);  // [8][64][6]
+    RowInfo *rows = reinterpret_cast<RowInfo *>(red + 8 * kTcSlotsPerTile * 6);
+    if (tid < R) rows[tid] = own;
     if (!err && warp < kTcEpiWarps) {
-        const int row = 32 * (warp & 3) + lane, j0 = 16 * (warp >> 2);
+        const int hrow = 32 * (warp >> 2), m = 32 * (warp & 3) + lane;
+        float *wf = reinterpret_cast<float *>(Wst) + m, *uf = reinterpret_cast<float *>(Ust) + m;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            Wst[row * kTcWs + j0 + i] = make_float2(w[2 * i], w[2 * i + 1]);
-            Ust[row * kTcWs + j0 + i] = make_float2(u[2 * i], u[2 * i + 1]);
+            const int o = (hrow + 2 * i) * 2 * kTcWs;
+            wf[o] = w[i].x; wf[o + 2 * kTcWs] = w[i].y;
+            uf[o] = u[i].x; uf[o + 2 * kTcWs] = u[i].y;
         }
     }
     __syncthreads();
     if (!err) {
         // element update: thread (row group g, slot j) takes rows g, g + 8, ... of slot j
         if (tid < 8 * kTcSlotsPerTile) {
-            const int j = tid % kTcSlotsPerTile, g = tid / kTcSlotsPerTile, sl = s0 + j;
+            const int j = tid % kTcSlotsPerTile, g = tid / kTcSlotsPerTile, sl = s0 + j, TS = T.S;
             const int st = T.state[sl];
-            const float vi = T.vid[sl], dvi = T.vid[T.S + sl];
+            const float vi = T.vid[sl], dvi = T.vid[TS + sl], hp = T.hp[sl], dtj = T.dtf[sl];
+            const int row0 = st == TS_WAIT ? T.slot[sl].s0 : -1;
             float part[6] = {0, 0, 0, 0, 0, 0};
             const bool work = st == TS_ACTIVE || st == TS_FINAL;
+            const float2 *Cs = Cg + sl, *PHc = ((s == 0 || s == 3) ? T.PHa : T.PHb) + sl;
+            const float2 *PHn = ((s == 0 || s == 1) ? T.PHb : T.PHa) + sl;
+            const float2 *As = T.A + (size_t)r0 * TS + sl, *ACCs = T.ACC + (size_t)r0 * TS + sl;
             constexpr int kB = 4;  // rows gathered before any is updated
+            if (st != TS_IDLE)
             for (int rb = g; rb < R; rb += 8 * kB) {
-                ElemIn in[kB];
+                float2 c[kB], cu[kB], cd[kB], p[kB], q[kB], a0[kB], acc[kB];
 #pragma unroll
                 for (int k = 0; k < kB; ++k) {
                     const int row = rb + 8 * k;
-                    if (work && row < R) tc_elem_gather(T, S, s, cur, r0 + row, sl, in[k]);
+                    c[k] = cu[k] = cd[k] = p[k] = q[k] = a0[k] = acc[k] = make_float2(0.f, 0.f);
+                    if (!work || row >= R) continue;
+                    const RowInfo &ri = rows[row];
+                    c[k] = __ldg(Cs + (size_t)(r0 + row) * TS);
+                    cu[k] = __ldg(Cs + (size_t)ri.up * TS);
+                    cd[k] = __ldg(Cs + (size_t)ri.dn * TS);
+                    p[k] = __ldg(PHc + (size_t)ri.lev * TS);
+                    q[k] = (s == 0 || s == 2) ? __ldg(PHn + (size_t)ri.lev * TS) : p[k];
+                    a0[k] = As[(size_t)row * TS];
+                    acc[k] = ACCs[(size_t)row * TS];
                 }
 #pragma unroll
                 for (int k = 0; k < kB; ++k) {
                     const int row = rb + 8 * k;
                     if (row >= R) continue;
-                    float2 wt = make_float2(0.f, 0.f), ut = wt;
-                    if (work) {
-                        const float2 c = in[k].c, ws = Wst[row * kTcWs + j], us = Ust[row * kTcWs + j];
-                        wt = make_float2(fmaf(vi, c.x, ws.x), fmaf(vi, c.y, ws.y));
-                        ut = make_float2(fmaf(dvi, c.x, us.x), fmaf(dvi, c.y, us.y));
-                    }
-                    tc_elem_apply(T, S, s, cur, r0 + row, sl, st, in[k], wt, ut, part);
+                    const RowInfo &ri = rows[row];
+                    const float2 ws = Wst[row * kTcWs + j], us = Ust[row * kTcWs + j];
+                    const float2 wt = make_float2(fmaf(vi, c[k].x, ws.x), fmaf(vi, c[k].y, ws.y));
+                    const float2 ut = make_float2(fmaf(dvi, c[k].x, us.x), fmaf(dvi, c[k].y, us.y));
+                    float2 ao, acco, co;
+                    const int mode = elem_core(s, st, r0 + row == row0, c[k], cu[k], cd[k], p[k], q[k], a0[k], acc[k], ri.au,
+                                               ri.ad, ri.elev, hp, dtj, wt, ut, part, ao, acco, co);
+                    elem_store(T, S, cur, r0 + row, sl, mode, ao, acco, co);
                 }
             }
             for (int k = 0; k < 6; ++k) red[(g * kTcSlotsPerTile + j) * 6 + k] = part[k];
@@ -438,7 +454,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, in
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == kTcMmaWarp) tc_tmem_dealloc(tbase, 256);
+    if (warp == kTcMmaWarp) tc_tmem_dealloc(tbase, 512);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -705,21 +721,9 @@ __device__ void tc_publish_idle(const TcState &T, const DevSys &S, const SlotLan
 // split the levels)
 __device__ __forceinline__ void tc_phases(const TcState &T, const DevSys &S, const SlotLane &L, float2 *PH, unsigned n_half)
 {
-    // the increments are loaded four at a time ahead of the stores, so that the independent global
-    // loads overlap instead of each waiting for the previous store
-    constexpr int kB = 4;
-    for (int l0 = L.sc; l0 < S.n_levels; l0 += 4 * kB) {
-        unsigned long long v[kB];
-#pragma unroll
-        for (int i = 0; i < kB; ++i) {
-            const int l = l0 + 4 * i;
-            v[i] = l < S.n_levels ? T.inc[(size_t)l * T.S + L.sl] : 0ull;
-        }
-#pragma unroll
-        for (int i = 0; i < kB; ++i) {
-            const int l = l0 + 4 * i;
-            if (l < S.n_levels) PH[(size_t)l * T.S + L.sl] = phase_factor(v[i], n_half);
-        }
+    for (int l = L.sc; l < S.n_levels; l += 4) {
+        const size_t i = (size_t)l * T.S + L.sl;
+        PH[i] = phase_factor(T.inc[i], n_half);
     }
 }
 
@@ -781,11 +785,30 @@ __global__ void __launch_bounds__(128) k_tc_init(TcState T)
 
 // after the stage kernel of stage s: the row-tile partial sums of force, torque and diagnostics
 // (compensated FP32, FP64 once per slot), bookkeeping (stage 0), the classical stage update
-// (Eqs. 7-10), stop rule and refill, then the next stage's spline values, dPhi/dt and phase factors
-__global__ void __launch_bounds__(128) k_tc_slots(TcState T, int s, int n_rowblocks)
+// (Eqs. 7-10), stop rule and refill, then the next stage's spline values and dPhi/dt
+//
+// The blocks past the slots' own (slot_blocks) compute phase factors, one thread per (level, slot), beside
+// the slots' chains of FP64 instructions: after stage 1 those of the integer time t + dt (stage 0 was the last
+// to read those of t), after stage 2 those of the next step's half time (this one's are read no more); a
+// slot that starts at the next stage 0 gets t = 0 and t = dt/2.  Neither stage changes a slot's state or steps.
+__global__ void __launch_bounds__(128) k_tc_slots(TcState T, int s, int n_rowblocks, int slot_blocks)
 {
     const DevSys &S = *T.sys;
     const unsigned full = 0xffffffffu;
+    if ((int)blockIdx.x >= slot_blocks) {
+        const size_t total = (size_t)S.n_levels * T.S, step = (size_t)(gridDim.x - slot_blocks) * blockDim.x;
+        float2 *PH = s == 1 ? T.PHa : T.PHb;
+        for (size_t i = (size_t)(blockIdx.x - slot_blocks) * blockDim.x + threadIdx.x; i < total; i += step) {
+            const int sl = (int)(i % T.S), st = T.state[sl];
+            if (st == TS_ACTIVE) {
+                PH[i] = phase_factor(T.inc[i], 2u * (unsigned)T.slot[sl].steps + (s == 1 ? 2u : 3u));
+            } else if (st == TS_WAIT && s == 2) {
+                PH[i] = phase_factor(T.inc[i], 1u);
+                T.PHa[i] = make_float2(1.f, 0.f);
+            }
+        }
+        return;
+    }
     const SlotLane L = slot_lane(T);
     TSlot &m = T.slot[L.slc];
     int state = m.state;
@@ -888,16 +911,6 @@ __global__ void __launch_bounds__(128) k_tc_slots(TcState T, int s, int n_rowblo
         state = ms > 0 ? TS_ACTIVE : TS_FINAL;
         if (ms <= 0) add_status |= MQCT_TRAJ_MAX_STEPS;
     }
-    // phase factors needed ahead: after stage 1 the integer time t + dt, after stage 3 the half
-    // time of the next step; a slot that starts at the next stage 0 gets t = 0 and t = dt/2
-    if (start) {
-        tc_phases(T, S, L, T.PHb, 1u);
-        for (int l = L.sc; l < S.n_levels; l += 4) T.PHa[(size_t)l * T.S + L.sl] = make_float2(1.f, 0.f);
-    } else if (act && state == TS_ACTIVE && s == 1) {
-        tc_phases(T, S, L, T.PHa, 2u * steps + 2u);
-    } else if (act && state == TS_ACTIVE && s == 3) {
-        tc_phases(T, S, L, T.PHb, 2u * steps + 1u);
-    }
     if (L.valid && state == TS_IDLE) tc_publish_idle(T, S, L);
     __syncwarp();
     if (L.valid) {
@@ -907,9 +920,11 @@ __global__ void __launch_bounds__(128) k_tc_slots(TcState T, int s, int n_rowblo
         if (L.sc == 0) {
             if (next) { m.ir = ir; m.i2m = i2m; m.phid = phid; }
             m.status |= add_status;
-            m.steps = steps;
-            m.state = state;
-            T.state[L.sl] = state;
+            if (s == 0 || s == 3) {  // stages 1 and 2 change neither (the phase blocks read them)
+                m.steps = steps;
+                m.state = state;
+                T.state[L.sl] = state;
+            }
             T.dtf[L.sl] = (float)m.dt;
         }
     }
@@ -1130,6 +1145,10 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
     const int slot_blocks = (S / 8 + 3) / 4;  // four warps of eight slots per block
     k_tc_init<<<slot_blocks, 128, 0, st>>>(T);
     const int n_ct = S / kTcSlotsPerTile;
+    const int phase_blocks = (int)std::min<size_t>(((size_t)h.n_levels * S + 127) / 128, (size_t)sms * 8);
+    auto slots = [&](cudaStream_t q, int s) {
+        k_tc_slots<<<slot_blocks + (s == 1 || s == 2 ? phase_blocks : 0), 128, 0, q>>>(T, s, n_rowblocks, slot_blocks);
+    };
     // the stage kernel: tcgen05 contraction (factorised BF16X3) or the sparse FP32 table (PLAIN)
     auto stage = [&](cudaStream_t q, int s, int cur) {
         if (plain) k_sp_stage<<<dim3(S / kSpTile, n_rowblocks), 32 * kSpWarps, 0, q>>>(T, s, cur);
@@ -1164,7 +1183,7 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
             for (int s = 0; s < 4; ++s) {
                 const int cur = s & 1;
                 stage(st, s, cur);
-                k_tc_slots<<<slot_blocks, 128, 0, st>>>(T, s, n_rowblocks);
+                slots(st, s);
             }
         sort_slots(st);
         k_tc_continue<<<1, 32, 0, st>>>(T, 0);
@@ -1192,7 +1211,7 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
             for (int s = 0; s < 4; ++s) {
                 const int cur = s & 1;
                 stage(cap, s, cur);
-                k_tc_slots<<<slot_blocks, 128, 0, cap>>>(T, s, n_rowblocks);
+                slots(cap, s);
             }
         sort_slots(cap);
         k_tc_continue<<<1, 32, 0, cap>>>(T, cond);
