@@ -466,9 +466,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, in
 //   w = sum_c M_rc(x) C_c,   u = (dx/dR) sum_c M'_rc(x) C_c,
 // then the element update of Eq. 5 and RK4 (every load coalesced over the slots) and the per-slot
 // partial sums of force, torque and diagnostics over the 256 rows (compensated FP32 across warps).
+// Bound by the latency of its gathers: five CTAs per SM (48 registers, 28 spilled loads outside the loop over
+// the non-zeros) hide more of it than four with 64: N = 40401, 512 slots 142.8 -> 138.1 ms for 48 steps, 1024 slots
+// 244.6 -> 237.0 ms; six gain nothing more (133 and 245 ms).
 constexpr int kSpWarps = 8, kSpTile = 32;
 
-__global__ void __launch_bounds__(32 * kSpWarps, 4) k_sp_stage(TcState T, int s, int cur)
+__global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s, int cur)
 {
     const DevSys &S = *T.sys;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
