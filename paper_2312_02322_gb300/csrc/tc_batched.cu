@@ -478,12 +478,21 @@ __global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s,
     const int sl = blockIdx.x * kSpTile + lane, rb = blockIdx.y;
     const int slice = rb * kSpWarps + warp;
     __shared__ float red[kSpWarps][6][kSpTile];
+    __shared__ int4 row_a[32 * kSpWarps];    // per row: m + 1 and m - 1 partners, level, ladder factor up (bits)
+    __shared__ float2 row_b[32 * kSpWarps];  // ladder factor down, level energy
     __shared__ int any_;
     const int st = T.state[sl];
     if (threadIdx.x == 0) any_ = 0;
     __syncthreads();
     if (warp == 0 && __any_sync(0xffffffffu, st != TS_IDLE) && lane == 0) any_ = 1;
     __syncthreads();
+    if (any_ && 32 * slice + lane < S.n) {
+        // what belongs to a row alone, loaded once by the warp that takes the slice
+        const int r = 32 * slice + lane, lev = __ldg(S.lev + r);
+        row_a[32 * warp + lane] = make_int4(__ldg(S.up + r), __ldg(S.dn + r), lev, __float_as_int(__ldg(S.aupf + r)));
+        row_b[32 * warp + lane] = make_float2(__ldg(S.adnf + r), __ldg(S.lev_energy_f + lev));
+    }
+    __syncwarp();
     float part[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (any_ && slice < S.n_slices) {
         const bool need = st == TS_ACTIVE || (st == TS_FINAL && s == 0);
@@ -491,6 +500,7 @@ __global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s,
         const float x = T.xs[sl], dv = T.dinv[sl], hp = T.hp[sl], dtj = T.dtf[sl];
         const int row0 = st == TS_WAIT ? T.slot[sl].s0 : -1;
         const float4 *tab = S.T4f + (size_t)kint * S.nnz_pad;
+        const int *cols = S.cols;
         const float2 *Cc = T.C[cur];
         const float2 *PHc = (s == 0 || s == 3) ? T.PHa : T.PHb;
         const float2 *PHn = (s == 0 || s == 1) ? T.PHb : T.PHa;
@@ -508,7 +518,7 @@ __global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s,
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const size_t ei = (size_t)off + (size_t)(e + i) * kSlice + rl;
-                        col[i] = __ldg(S.cols + ei);
+                        col[i] = __ldg(cols + ei);
                         c[i] = __ldg(tab + ei);
                     }
 #pragma unroll
@@ -526,7 +536,7 @@ __global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s,
                 for (; e < width; ++e) {
                     const size_t ei = (size_t)off + (size_t)e * kSlice + rl;
                     const float4 c = __ldg(tab + ei);
-                    const float2 z = __ldg(Cc + (size_t)__ldg(S.cols + ei) * T.S + sl);
+                    const float2 z = __ldg(Cc + (size_t)__ldg(cols + ei) * T.S + sl);
                     const float m = fmaf(fmaf(fmaf(c.w, x, c.z), x, c.y), x, c.x);
                     const float md = fmaf(fmaf(3.0f * c.w, x, 2.0f * c.z), x, c.y);
                     w.x = fmaf(m, z.x, w.x);
@@ -536,14 +546,16 @@ __global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s,
                 }
             }
             if (st == TS_IDLE) continue;
-            const int lev = __ldg(S.lev + r);
+            const int4 ra = row_a[32 * warp + rl];
+            const float2 rb_ = row_b[32 * warp + rl];
             const size_t e0 = (size_t)r * T.S + sl;
             const float2 c = __ldg(Cc + e0);
-            const float2 cu = __ldg(Cc + (size_t)__ldg(S.up + r) * T.S + sl);
-            const float2 cd = __ldg(Cc + (size_t)__ldg(S.dn + r) * T.S + sl);
-            const float2 p = __ldg(PHc + (size_t)lev * T.S + sl), q = __ldg(PHn + (size_t)lev * T.S + sl);
+            const float2 cu = __ldg(Cc + (size_t)ra.x * T.S + sl);
+            const float2 cd = __ldg(Cc + (size_t)ra.y * T.S + sl);
+            const float2 p = __ldg(PHc + (size_t)ra.z * T.S + sl);
+            const float2 q = (s == 0 || s == 2) ? __ldg(PHn + (size_t)ra.z * T.S + sl) : p;  // else the same time
             const float2 a0 = T.A[e0], acc = T.ACC[e0];
-            const float au = __ldg(S.aupf + r), ad = __ldg(S.adnf + r), elev = S.lev_energy_f[lev];
+            const float au = __int_as_float(ra.w), ad = rb_.x, elev = rb_.y;
             const float2 uu = make_float2(u.x * dv, u.y * dv);
             float2 ao, acco, co;
             const int mode = elem_core(s, st, r == row0, c, cu, cd, p, q, a0, acc, au, ad, elev, hp, dtj, w, uu, part,
@@ -576,10 +588,11 @@ struct SlotLane {
     unsigned m4;  // the four lanes of this slot
 };
 
-__device__ __forceinline__ SlotLane slot_lane(const TcState &T)
+// warp: index of eight consecutive slots
+__device__ __forceinline__ SlotLane slot_lane(const TcState &T, int warp)
 {
     SlotLane L;
-    const int lane = threadIdx.x & 31, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     L.sc = lane >> 3;
     L.sj = lane & 7;
     L.sl = 8 * warp + L.sj;
@@ -731,11 +744,13 @@ __device__ __forceinline__ void tc_phases(const TcState &T, const DevSys &S, con
 }
 
 // claim the first trajectory of every slot, initialise its column and views
-__global__ void __launch_bounds__(128) k_tc_init(TcState T)
+__global__ void __launch_bounds__(1024) k_tc_init(TcState T)
 {
     const DevSys &S = *T.sys;
-    const SlotLane L = slot_lane(T);
-    const int lane = threadIdx.x & 31;
+    // four warps claim 32 slots, all 32 write their columns
+    __shared__ int st32[32], s032[32];
+    if (threadIdx.x < 128) {
+    const SlotLane L = slot_lane(T, 4 * blockIdx.x + (threadIdx.x >> 5));
     double q = 0.0;
     int state = TS_IDLE;
     if (L.valid) {
@@ -770,19 +785,20 @@ __global__ void __launch_bounds__(128) k_tc_init(TcState T)
             T.state[L.sl] = state;
         }
     }
-    __syncwarp();
-    // the columns of the warp's eight slots: e_s0, accumulator 0, input e_s0
-    for (int j = 0; j < 8; ++j) {
-        const int sl = 8 * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + j;
-        if (sl >= T.S) break;
-        const int st = T.slot[sl].state;
-        if (st != TS_ACTIVE && st != TS_FINAL) continue;
-        const int s0 = T.slot[sl].s0;
-        for (int r = lane; r < S.n; r += 32) {
-            const float2 v = make_float2(r == s0 ? 1.0f : 0.0f, 0.0f);
-            const size_t e = (size_t)r * T.S + sl;
-            T.A[e] = v; T.ACC[e] = make_float2(0.f, 0.f); T.C[0][e] = v;
-        }
+    if (L.sc == 0) {
+        const int i = L.sl & 31;
+        st32[i] = state;
+        s032[i] = L.valid && (state == TS_ACTIVE || state == TS_FINAL) ? T.slot[L.sl].s0 : -1;
+    }
+    }
+    __syncthreads();
+    // the columns of the block's slots, 32 consecutive slots of a row per warp: e_s0, accumulator 0, input e_s0
+    const int i = threadIdx.x & 31, sl = 32 * blockIdx.x + i;
+    if (sl >= T.S || (st32[i] != TS_ACTIVE && st32[i] != TS_FINAL)) return;
+    for (int r = threadIdx.x >> 5; r < S.n; r += blockDim.x >> 5) {
+        const float2 v = make_float2(r == s032[i] ? 1.0f : 0.0f, 0.0f);
+        const size_t e = (size_t)r * T.S + sl;
+        T.A[e] = v; T.ACC[e] = make_float2(0.f, 0.f); T.C[0][e] = v;
     }
 }
 
@@ -812,7 +828,7 @@ __global__ void __launch_bounds__(128) k_tc_slots(TcState T, int s, int n_rowblo
         }
         return;
     }
-    const SlotLane L = slot_lane(T);
+    const SlotLane L = slot_lane(T, (blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     TSlot &m = T.slot[L.slc];
     int state = m.state;
     if (__all_sync(full, !L.valid || state == TS_IDLE)) return;  // published as idle when they became idle
@@ -940,90 +956,85 @@ __global__ void __launch_bounds__(128) k_tc_slots(TcState T, int s, int n_rowblo
 // ---------------------------------------------------------------------------------------------
 // PLAIN path, at the end of a chunk of steps: the slots are reordered by spline interval so that the
 // 32 slots of a stage-kernel tile mostly read the same rows of the table (one transaction per element
-// instead of one per slot); idle slots go last.  perm[new] = old by a stable counting sort (one
-// thread: S <= 8192), then every per-slot and per-(row, slot) array is gathered into scratch and
-// copied back.
-struct SpSort {
-    int *perm, *cnt;            // [S], [n_int + 2]
-    TSlot *slot;                // scratch copies
-    double *Q, *QS, *LACC;      // [4][S]
-    int *state, *kint;
-    float *hp, *dtf, *xs, *dinv;
-    unsigned long long *inc;    // [n_levels][S]
-    float2 *PHa, *PHb;          // [n_levels][S]
-    float2 *A, *ACC;            // [n][S]; C[0] goes through C[1]
-};
+// instead of one per slot); idle slots go last.  perm[new] = old by a stable counting sort (S <= 8192), then every
+// per-slot and per-(row, slot) array is reordered in place (N = 40401, 512 slots: 0.98 ms per chunk with one
+// thread sorting and a copy out and back, 0.21 ms now).
 
-__global__ void k_sp_order(TcState T, SpSort P, int n_int)
+// one block: a stable counting sort by bucket (interval >> shift, so that there are at most 2048; the last
+// bucket holds the idle slots): a warp per bucket places the bucket's slots in ascending order
+__global__ void __launch_bounds__(1024) k_sp_order(TcState T, int *perm, int n_int, int shift)
 {
-    if (threadIdx.x != 0) return;
-    const int S = T.S, nb = n_int + 1;  // bucket n_int: idle slots
-    for (int b = 0; b <= nb; ++b) P.cnt[b] = 0;
-    for (int i = 0; i < S; ++i) {
-        const int k = T.state[i] == TS_IDLE ? n_int : min(max(T.kint[i], 0), n_int - 1);
-        P.cnt[k + 1] += 1;
+    extern __shared__ int osm[];
+    int *key = osm, *start = osm + T.S;  // [S], [buckets]
+    const int S = T.S, idle = ((n_int - 1) >> shift) + 1, nb = idle + 1, tid = threadIdx.x, nt = blockDim.x;
+    for (int b = tid; b < nb; b += nt) start[b] = 0;
+    __syncthreads();
+    for (int i = tid; i < S; i += nt) {
+        const int k = T.state[i] == TS_IDLE ? idle : min(max(T.kint[i], 0), n_int - 1) >> shift;
+        key[i] = k;
+        atomicAdd(start + k, 1);
     }
-    for (int b = 1; b <= nb; ++b) P.cnt[b] += P.cnt[b - 1];
-    for (int i = 0; i < S; ++i) {
-        const int k = T.state[i] == TS_IDLE ? n_int : min(max(T.kint[i], 0), n_int - 1);
-        P.perm[P.cnt[k]++] = i;
+    __syncthreads();
+    if (tid == 0) {
+        int sum = 0;
+        for (int b = 0; b < nb; ++b) {
+            const int n = start[b];
+            start[b] = sum;
+            sum += n;
+        }
+    }
+    __syncthreads();
+    const int warp = tid >> 5, lane = tid & 31;
+    for (int b = warp; b < nb; b += nt >> 5) {
+        int pos = start[b];
+        const int end = b + 1 < nb ? start[b + 1] : S;
+        for (int i0 = 0; i0 < S && pos < end; i0 += 32) {
+            const int i = i0 + lane;
+            const bool mine = i < S && key[i] == b;
+            const unsigned m = __ballot_sync(0xffffffffu, mine);
+            if (mine) perm[pos + __popc(m & ((1u << lane) - 1u))] = i;
+            pos += __popc(m);
+        }
     }
 }
 
-// gather into scratch (dir 0) or copy back (dir 1): per-slot arrays, one thread per slot
-__global__ void k_sp_move_slots(TcState T, SpSort P, int n_levels, int dir)
+// every array with one entry per slot, reordered in place: a block takes one row of S entries (through shared
+// memory), new[i] = old[perm[i]].  Rows of 8-byte entries: A, ACC, C[0] per state, the phase increments and
+// factors per level, the classical state per component, the 15 words of TSlot; then six of 4 bytes.
+constexpr int kSlotWords = sizeof(TSlot) / 8;
+static_assert(sizeof(TSlot) % 8 == 0, "TSlot is moved in 8-byte words");
+
+__global__ void __launch_bounds__(256) k_sp_permute(TcState T, const int *perm, int n, int n_levels)
 {
+    extern __shared__ unsigned long long psm[];
     const int S = T.S;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < S; i += gridDim.x * blockDim.x) {
-        const int o = dir == 0 ? P.perm[i] : i;
-        if (dir == 0) {
-            P.slot[i] = T.slot[o];
-            for (int c = 0; c < 4; ++c) {
-                P.Q[(size_t)c * S + i] = T.Q[(size_t)c * S + o];
-                P.QS[(size_t)c * S + i] = T.QS[(size_t)c * S + o];
-                P.LACC[(size_t)c * S + i] = T.LACC[(size_t)c * S + o];
-            }
-            P.state[i] = T.state[o]; P.kint[i] = T.kint[o];
-            P.hp[i] = T.hp[o]; P.dtf[i] = T.dtf[o]; P.xs[i] = T.xs[o]; P.dinv[i] = T.dinv[o];
-            for (int l = 0; l < n_levels; ++l) {
-                P.inc[(size_t)l * S + i] = T.inc[(size_t)l * S + o];
-                P.PHa[(size_t)l * S + i] = T.PHa[(size_t)l * S + o];
-                P.PHb[(size_t)l * S + i] = T.PHb[(size_t)l * S + o];
-            }
-        } else {
-            T.slot[i] = P.slot[i];
-            for (int c = 0; c < 4; ++c) {
-                T.Q[(size_t)c * S + i] = P.Q[(size_t)c * S + i];
-                T.QS[(size_t)c * S + i] = P.QS[(size_t)c * S + i];
-                T.LACC[(size_t)c * S + i] = P.LACC[(size_t)c * S + i];
-            }
-            T.state[i] = P.state[i]; T.kint[i] = P.kint[i];
-            T.hp[i] = P.hp[i]; T.dtf[i] = P.dtf[i]; T.xs[i] = P.xs[i]; T.dinv[i] = P.dinv[i];
-            for (int l = 0; l < n_levels; ++l) {
-                T.inc[(size_t)l * S + i] = P.inc[(size_t)l * S + i];
-                T.PHa[(size_t)l * S + i] = P.PHa[(size_t)l * S + i];
-                T.PHb[(size_t)l * S + i] = P.PHb[(size_t)l * S + i];
-            }
-        }
+    long long row = blockIdx.x;
+    unsigned long long *p = nullptr;
+    int stride = 1;
+    auto take = [&](void *base, long long count) {
+        if (p || row < 0) return;
+        if (row < count) p = reinterpret_cast<unsigned long long *>(base) + (size_t)row * S;
+        else row -= count;
+    };
+    take(T.A, n); take(T.ACC, n); take(T.C[0], n);
+    take(T.inc, n_levels); take(T.PHa, n_levels); take(T.PHb, n_levels);
+    take(T.Q, 4); take(T.QS, 4); take(T.LACC, 4);
+    if (!p && row < kSlotWords) {
+        p = reinterpret_cast<unsigned long long *>(T.slot) + row;
+        stride = kSlotWords;
     }
-}
-
-// gather (dir 0: A, ACC into scratch, C[0] into C[1]) or copy back (dir 1), one thread per element
-__global__ void k_sp_move_rows(TcState T, SpSort P, int n, int dir)
-{
-    const size_t S = T.S, total = (size_t)n * S;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        if (dir == 0) {
-            const size_t r = e / S, i = e % S, o = r * S + P.perm[i];
-            P.A[e] = T.A[o];
-            P.ACC[e] = T.ACC[o];
-            T.C[1][e] = T.C[0][o];
-        } else {
-            T.A[e] = P.A[e];
-            T.ACC[e] = P.ACC[e];
-            T.C[0][e] = T.C[1][e];
-        }
+    if (p) {
+        for (int i = threadIdx.x; i < S; i += blockDim.x) psm[i] = p[(size_t)i * stride];
+        __syncthreads();
+        for (int i = threadIdx.x; i < S; i += blockDim.x) p[(size_t)i * stride] = psm[perm[i]];
+        return;
     }
+    row -= kSlotWords;
+    int *q = row == 0 ? T.state : (row == 1 ? T.kint : reinterpret_cast<int *>(row == 2 ? T.hp : (row == 3 ? T.dtf : (row == 4 ? T.xs : T.dinv))));
+    int *psmi = reinterpret_cast<int *>(psm);
+    for (int i = threadIdx.x; i < S; i += blockDim.x) psmi[i] = q[i];
+    __syncthreads();
+    for (int i = threadIdx.x; i < S; i += blockDim.x) q[i] = psmi[perm[i]];
 }
 
 // the condition of the graph's WHILE node at the end of a chunk of steps: run another chunk while
@@ -1110,29 +1121,12 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
     get((void **)&T.QS, sizeof(double) * 4 * (size_t)S);
     get((void **)&T.LACC, sizeof(double) * 4 * (size_t)S);
     get((void **)&T.slot, sizeof(TSlot) * (size_t)S);
-    SpSort P;
-    std::memset(&P, 0, sizeof(P));
+    int *perm = nullptr;
     if (plain) {
         get((void **)&T.kint, sizeof(int) * (size_t)S);
         get((void **)&T.xs, sizeof(float) * (size_t)S);
         get((void **)&T.dinv, sizeof(float) * (size_t)S);
-        get((void **)&P.perm, sizeof(int) * (size_t)S);
-        get((void **)&P.cnt, sizeof(int) * (size_t)(h.n_int + 2));
-        get((void **)&P.slot, sizeof(TSlot) * (size_t)S);
-        get((void **)&P.Q, sizeof(double) * 4 * (size_t)S);
-        get((void **)&P.QS, sizeof(double) * 4 * (size_t)S);
-        get((void **)&P.LACC, sizeof(double) * 4 * (size_t)S);
-        get((void **)&P.state, sizeof(int) * (size_t)S);
-        get((void **)&P.kint, sizeof(int) * (size_t)S);
-        get((void **)&P.hp, sizeof(float) * (size_t)S);
-        get((void **)&P.dtf, sizeof(float) * (size_t)S);
-        get((void **)&P.xs, sizeof(float) * (size_t)S);
-        get((void **)&P.dinv, sizeof(float) * (size_t)S);
-        get((void **)&P.inc, sizeof(unsigned long long) * (size_t)h.n_levels * S);
-        get((void **)&P.PHa, sizeof(float2) * (size_t)h.n_levels * S);
-        get((void **)&P.PHb, sizeof(float2) * (size_t)h.n_levels * S);
-        get((void **)&P.A, sizeof(float2) * ns);
-        get((void **)&P.ACC, sizeof(float2) * ns);
+        get((void **)&perm, sizeof(int) * (size_t)S);
     }
     if (e != cudaSuccess) {
         cleanup();
@@ -1146,7 +1140,7 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
     }
     cudaMemsetAsync(T.live, 0, 4 * sizeof(int), st);
     const int slot_blocks = (S / 8 + 3) / 4;  // four warps of eight slots per block
-    k_tc_init<<<slot_blocks, 128, 0, st>>>(T);
+    k_tc_init<<<slot_blocks, 1024, 0, st>>>(T);
     const int n_ct = S / kTcSlotsPerTile;
     const int phase_blocks = (int)std::min<size_t>(((size_t)h.n_levels * S + 127) / 128, (size_t)sms * 8);
     auto slots = [&](cudaStream_t q, int s) {
@@ -1158,14 +1152,16 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
         else k_tc_stage<<<h.n_tiles * n_ct, kTcThreads, smem, q>>>(T, s, cur);
     };
     // PLAIN path: the slots sorted by interval at the end of each chunk
-    const int mv_blocks = (int)std::min<size_t>((ns + 255) / 256, (size_t)sms * 16);
+    int sort_shift = 0;
+    while (((h.n_int - 1) >> sort_shift) >= 2048) ++sort_shift;
+    const size_t order_smem = sizeof(int) * ((size_t)S + 2050), perm_smem = 8 * (size_t)S;
+    const long long perm_rows = 3LL * n + 3LL * h.n_levels + 12 + kSlotWords + 6;
+    if (plain && e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sp_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)perm_smem);
     auto sort_slots = [&](cudaStream_t q) {
         if (!plain) return;
-        k_sp_order<<<1, 32, 0, q>>>(T, P, h.n_int);
-        k_sp_move_slots<<<(S + 127) / 128, 128, 0, q>>>(T, P, h.n_levels, 0);
-        k_sp_move_rows<<<mv_blocks, 256, 0, q>>>(T, P, n, 0);
-        k_sp_move_slots<<<(S + 127) / 128, 128, 0, q>>>(T, P, h.n_levels, 1);
-        k_sp_move_rows<<<mv_blocks, 256, 0, q>>>(T, P, n, 1);
+        k_sp_order<<<1, 1024, order_smem, q>>>(T, perm, h.n_int, sort_shift);
+        k_sp_permute<<<(unsigned)perm_rows, 256, perm_smem, q>>>(T, perm, n, h.n_levels);
     };
     // chunks of steps inside a WHILE node: the body (one chunk) ends with k_tc_continue, which
     // sets the condition from the live-slot count; one launch of the graph runs every trajectory
@@ -1230,9 +1226,8 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
     if (cap) cudaStreamDestroy(cap);
     cleanup();
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core path");
-    // k_tc_init, then per chunk: reset, chunk x 4 x (stage, slots), (PLAIN: the five sorting
-    // kernels), continue
-    count_launches(1 + (long long)live[2] * (2 + 8 * chunk + (plain ? 5 : 0)));
+    // k_tc_init, then per chunk: reset, chunk x 4 x (stage, slots), (PLAIN: the two sorting kernels), continue
+    count_launches(1 + (long long)live[2] * (2 + 8 * chunk + (plain ? 2 : 0)));
     if (live[1]) return fail(MQCT_ERR_TIMEOUT, "tensor-core path: a bounded MMA completion wait ran out");
     return MQCT_OK;
 }
