@@ -316,8 +316,8 @@ __device__ __forceinline__ double reduce16(double (&v)[16], int lane)
 // enter the result as conj(p) M (i z - PPhibar Dc) only and are contracted as that one vector; the sums
 // Re(kbar^dag (-i conj(p) M' c)), Re(c^dag M'' c) and Re((Dc)^dag M' c) follow from the per-term sums alpha, beta, gamma
 // that the parameters need anyway; those are reduced five terms at a time (reduce16).  N = 441, 128 trajectories,
-// with the forward stage in one pass and the kept stage states: 1169 -> 695 ms.  The mixed form below keeps the
-// order of its sums, and with it its bits.
+// with the forward stage in one pass and the kept stage states: 1169 -> 695 ms (601
+// without the counting propagation).  The mixed form below keeps the order of its sums, and with it its bits.
 __device__ void vjp_eval64(const DevSys &S, double t, const double2 *Ya, const double *Yq, AdjSmem<double> &m,
                            AdjCtl<double> &c, double *wred)
 {
@@ -616,7 +616,7 @@ __device__ void vjp_eval32(const DevSys &S, double t, unsigned n_half, const flo
 
 // two CTAs per SM in the mixed precision, whose barriers and chains then fill each other's gaps (its FP64
 // counterpart fills the FP64 pipe and its shared memory with one): N = 441, 256 trajectories 498 -> 313 ms together
-// with the kept stage states
+// with the kept stage states (286 without the counting propagation)
 template <class R>
 __global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 2 : 1) k_adjoint(AdjArgs a)
 {
@@ -939,16 +939,22 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
             !(t.b >= 0) || !(t.r0 > t.b) || t.max_steps < 0 || !std::isfinite(t.r_end))
             return fail(MQCT_ERR_INVALID_ARG, "mqct_adjoint: invalid trajectory");
     }
-    // forward step counts bound the checkpoint storage
-    std::vector<mqct_diag> dg(n);
+    // what the forward propagation refuses, the adjoint refuses (one trajectory of no steps)
     {
         mqct_system one = sys;
-        mqct_status s2 = mqct_propagate(&one, 1, ht.data(), n, nullptr, nullptr, dg.data(), cuda_stream);
+        mqct_traj t0 = ht[0];
+        mqct_diag d0;
+        t0.max_steps = 0;
+        const mqct_status s2 = mqct_propagate(&one, 1, &t0, 1, nullptr, nullptr, &d0, cuda_stream);
         if (s2 != MQCT_OK && s2 != MQCT_ERR_TRAJ) return s2;
     }
-    int max_steps = 1;
-    for (auto &d : dg) max_steps = std::max(max_steps, d.steps);
-    const int max_ckpt = max_steps / ckpt + 2;
+    // Checkpoint storage: three free flights 2 r0 / v of every trajectory, at most its max_steps.  A trajectory
+    // that outruns it (an orbiting one; status CKPT) makes the call count the steps by a forward propagation and
+    // run again; so does storage above 4 GB, before the first run.  N = 441, against a counting propagation in
+    // every call: FP64, 128 trajectories, 695 -> 601 ms; mixed, 256 trajectories, 313 -> 286.
+    double bound = 1.0;
+    for (const mqct_traj &t : ht)
+        bound = std::max(bound, std::min((double)t.max_steps, 64.0 + 6.0 * t.r0 / (t.dt * std::sqrt(2.0 * t.e_coll / h.mu))));
     // a stored state: amplitudes (FP32: and their compensation terms), then 4 classical doubles
     const size_t rsz = fp32 ? sizeof(float) : sizeof(double);
     const size_t amp_bytes = ((fp32 ? 4 : 2) * (size_t)h.n * rsz + 15) & ~(size_t)15;
@@ -976,6 +982,23 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, smem)) != cudaSuccess)
         return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     const int grid = std::max(1, std::min(n, sms * std::max(per_sm, 1)));
+    auto count_steps = [&](int &steps) -> mqct_status {
+        std::vector<mqct_diag> dg(n);
+        mqct_system one = sys;
+        const mqct_status s2 = mqct_propagate(&one, 1, ht.data(), n, nullptr, nullptr, dg.data(), cuda_stream);
+        if (s2 != MQCT_OK && s2 != MQCT_ERR_TRAJ) return s2;
+        steps = 1;
+        for (auto &d : dg) steps = std::max(steps, d.steps);
+        return MQCT_OK;
+    };
+    int max_steps = 0;
+    bool counted = (bound / ckpt + 2.0) * (double)grid * (double)stride > 4.0 * (1ull << 30);
+    if (counted) {
+        const mqct_status s2 = count_steps(max_steps);
+        if (s2 != MQCT_OK) return s2;
+    } else {
+        max_steps = (int)bound;
+    }
     const bool stages = (size_t)grid * ckpt * (stride + stage_bytes) <= (size_t)16 << 30;
     const size_t seg_stride = stride + (stages ? stage_bytes : 0);
     std::vector<void *> tmp;
@@ -1008,14 +1031,13 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         return cuda_fail(e, "staging");
     }
     aa.dLds = (const double *)ptr;
-    aa.n = n; aa.n_groups = n_groups; aa.K = ckpt; aa.max_ckpt = max_ckpt; aa.stride = stride;
+    aa.n = n; aa.n_groups = n_groups; aa.K = ckpt; aa.stride = stride;
     aa.seg_stride = seg_stride; aa.stages = stages ? 1 : 0;
     int *queue = nullptr;
-    unsigned char *scratch = nullptr, *vec = nullptr;
+    unsigned char *vec = nullptr;
     double *theta = nullptr, *out = nullptr;
     int *status = nullptr;
     if ((e = get((void **)&queue, sizeof(int))) != cudaSuccess ||
-        (e = get((void **)&scratch, (size_t)grid * ((size_t)max_ckpt * stride + (size_t)ckpt * seg_stride))) != cudaSuccess ||
         (vec_global && (e = get((void **)&vec, (size_t)grid * vec_bytes)) != cudaSuccess) ||
         (e = get((void **)&theta, sizeof(double) * (size_t)n * h.P)) != cudaSuccess ||
         (e = get((void **)&status, sizeof(int) * (size_t)n)) != cudaSuccess ||
@@ -1023,19 +1045,41 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         cleanup();
         return cuda_fail(e, "cudaMallocAsync (adjoint scratch)");
     }
-    aa.queue = queue; aa.scratch = scratch; aa.theta_traj = theta; aa.status = status;
+    aa.queue = queue; aa.theta_traj = theta; aa.status = status;
     aa.vec = vec; aa.vec_bytes = vec_bytes;
-    cudaMemsetAsync(queue, 0, sizeof(int), st);
-    if (fp32) k_adjoint<float><<<grid, kAdjThreads, smem, st>>>(aa);
-    else k_adjoint<double><<<grid, kAdjThreads, smem, st>>>(aa);
-    k_sum_theta<<<(h.P + 63) / 64, 64, 0, st>>>(theta, n, h.P, out);
-    count_launches(2);
-    if ((e = cudaGetLastError()) != cudaSuccess) { cleanup(); return cuda_fail(e, "adjoint kernels"); }
     std::vector<int> hst(n);
-    e = cudaMemcpyAsync(dL_dparam, out, sizeof(double) * h.P, adj_is_dev(dL_dparam) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hst.data(), status, sizeof(int) * n, cudaMemcpyDeviceToHost, st);
+    int launches = 0;
+    for (;;) {
+        aa.max_ckpt = max_steps / ckpt + 2;
+        void *scratch = nullptr;
+        if ((e = cudaMallocAsync(&scratch, (size_t)grid * ((size_t)aa.max_ckpt * stride + (size_t)ckpt * seg_stride), st)) != cudaSuccess) {
+            cleanup();
+            return cuda_fail(e, "cudaMallocAsync (adjoint checkpoints)");
+        }
+        aa.scratch = static_cast<unsigned char *>(scratch);
+        cudaMemsetAsync(queue, 0, sizeof(int), st);
+        if (fp32) k_adjoint<float><<<grid, kAdjThreads, smem, st>>>(aa);
+        else k_adjoint<double><<<grid, kAdjThreads, smem, st>>>(aa);
+        launches += 1;
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(hst.data(), status, sizeof(int) * n, cudaMemcpyDeviceToHost, st);
+        cudaFreeAsync(scratch, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "adjoint kernels"); }
+        bool outran = false;
+        for (int i = 0; i < n; ++i) outran |= (hst[i] & MQCT_TRAJ_CKPT) != 0;
+        if (counted || !outran) break;
+        const mqct_status s2 = count_steps(max_steps);
+        if (s2 != MQCT_OK) { cleanup(); return s2; }
+        counted = true;
+    }
+    k_sum_theta<<<(h.P + 63) / 64, 64, 0, st>>>(theta, n, h.P, out);
+    count_launches(launches + 1);
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(dL_dparam, out, sizeof(double) * h.P, adj_is_dev(dL_dparam) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
     cleanup();
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync");
+    if (e != cudaSuccess) return cuda_fail(e, "adjoint sums");
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     for (int i = 0; i < n; ++i)
         if (hst[i] != 0 && hst[i] != MQCT_TRAJ_TABLE_RANGE)
