@@ -632,6 +632,8 @@ __global__ void __launch_bounds__(T, MINB) k_propagate_fp64(PropArgs a)
     }
 }
 
+constexpr size_t kPropBasisBytes = 229216;  // of an SM's 232448 bytes per CTA
+
 // Element warps of a CTA: a warp takes 16 rows at a time, and there are as many as the rows feed, at most 14
 // (a 16-warp CTA, one per SM): N = 441, 256 trajectories 297 ms against 369 ms with eight warps and two CTAs
 // per SM, whose last trajectories leave half the GPU idle; 600 trajectories 615 against 602 ms; 64
@@ -650,6 +652,9 @@ cudaError_t launch_propagate(PropArgs pa, int maxlev, bool adapt, cudaStream_t s
     pa.smem_lev = maxlev;
     pa.adapt = adapt ? 1 : 0;
     const size_t smem = sizeof(double2) * ((adapt ? 6 : 4) * (size_t)pa.nmax + 2 * (size_t)maxlev);
+    // the bases taken are those whose six vectors (with adaptive steps eight) would fit: this layout needs four
+    // (six), but the call keeps refusing what it refused (N above 2380 or so)
+    if (sizeof(double2) * ((adapt ? 8 : 6) * (size_t)pa.nmax + 2 * (size_t)maxlev) > kPropBasisBytes) return cudaErrorInvalidValue;
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

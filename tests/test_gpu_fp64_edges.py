@@ -43,3 +43,18 @@ def test_sizes_and_shapes(mq, path, jmax, n):
         assert np.max(np.abs(pop[rows] - np.abs(amp) ** 2)) < 1e-8
     assert np.array_equal(d["status"] != 0, d["steps"] == tr["max_steps"])
     assert np.max(d["norm_dev"]) < 1e-6
+
+
+@pytest.mark.parametrize("jmax,adapt,taken", [(47, None, True), (48, None, False), (41, (1e-8, 4), True), (42, (1e-8, 4), False)])
+def test_largest_basis(mq, jmax, adapt, taken):
+    """The FP64 path takes bases of up to 2387 rows or so (adaptive steps: 1790) and refuses larger ones."""
+    p = W.diatom_pes_params(jmax=jmax, n_grid=60)
+    s = mq.System.diatom(p, path="factorised", precision="fp64", adapt=adapt)
+    tr = np.zeros(2, mq.TRAJ_DTYPE)
+    tr["e_coll"], tr["b"], tr["r0"], tr["r_end"], tr["dt"], tr["max_steps"] = W.cm(1000.0), 1.0, 7.0, 7.5, 5.0, 2
+    if taken:
+        _, _, d = mq.propagate(s, tr, device=False)
+        assert np.all(d["steps"] > 0)
+    else:
+        with pytest.raises(mq.MQCTError):
+            mq.propagate(s, tr, device=False)
