@@ -953,15 +953,23 @@ __global__ void __launch_bounds__(T, batched_min_blocks<T>()) k_batched_f32(Batc
     }
 }
 
-// the largest slot count (4, 8, 16 or 32, at most BMAX) with which a system fits a CTA of the shape
-// in `cap` bytes of shared memory; 0 if none
+// the largest slot count (4, 8, 16 or 32, at most BMAX) with which a system fits a CTA of the shape; 0 if
+// none.  The first bound (`cap` bytes for three amplitude arrays, two values per term and slot and eight
+// partial sums) says which bases a shape takes, whatever the layout, so that a shape that a caller keeps
+// stays valid; the layout above it is at most 16 L B bytes larger, which fits for every such basis with
+// four slots.
 template <int BMAX, int T, int kUpt>
 int batched_slots(const DevSys &h, size_t cap)
 {
-    constexpr int TE = (T / 32 - batch_slot_warps(BMAX)) * 32;
-    for (int b = BMAX; b >= 4; b >>= 1)
-        if ((size_t)h.n * (b / 4) <= (size_t)kUpt * TE && batched_smem<BMAX, T, kUpt>(h, b) + sizeof(BatchShared<BMAX>) <= cap)
+    constexpr int NE = T / 32 - batch_slot_warps(BMAX);
+    constexpr size_t kMaxBytes = 232448;  // shared memory of a CTA
+    const size_t n = h.n, nl = h.n_levels, L = h.L;
+    for (int b = BMAX; b >= 4; b >>= 1) {
+        const size_t bound = 24 * (n + nl) * b + 16 * L * b + 4 * nl + 32 * (size_t)NE * b + 16 + 400 + 200 * BMAX;
+        if (n * (b / 4) <= (size_t)kUpt * NE * 32 && bound <= cap &&
+            batched_smem<BMAX, T, kUpt>(h, b) + sizeof(BatchShared<BMAX>) <= kMaxBytes)
             return b;
+    }
     return 0;
 }
 
