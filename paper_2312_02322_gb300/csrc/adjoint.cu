@@ -1052,7 +1052,20 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     for (;;) {
         aa.max_ckpt = max_steps / ckpt + 2;
         void *scratch = nullptr;
-        if ((e = cudaMallocAsync(&scratch, (size_t)grid * ((size_t)aa.max_ckpt * stride + (size_t)ckpt * seg_stride), st)) != cudaSuccess) {
+        e = cudaMallocAsync(&scratch, (size_t)grid * ((size_t)aa.max_ckpt * stride + (size_t)ckpt * aa.seg_stride), st);
+        if (e == cudaErrorMemoryAllocation && (aa.stages || !counted)) {
+            // short of memory: the least that the call can do with, no stage states and counted steps
+            cudaGetLastError();
+            aa.stages = 0;
+            aa.seg_stride = stride;
+            if (!counted) {
+                const mqct_status s2 = count_steps(max_steps);
+                if (s2 != MQCT_OK) { cleanup(); return s2; }
+                counted = true;
+            }
+            continue;
+        }
+        if (e != cudaSuccess) {
             cleanup();
             return cuda_fail(e, "cudaMallocAsync (adjoint checkpoints)");
         }
