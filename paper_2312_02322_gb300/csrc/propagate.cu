@@ -24,7 +24,7 @@
 // the passes are ordered for the fewest FP64 instructions, and no chain of them runs while the
 // element warps wait.  Measured against a kernel that wrote w to shared memory for a second pass (two
 // barriers and one thread's FP64 chain per stage): N = 49, 32 trajectories 34 -> 12 us per step; N = 441 PLAIN, 256
-// trajectories 471 -> 297 ms (FP64 pipe 75 -> 93 % busy, 14 % fewer FP64 instructions, 15 % fewer padded
+// trajectories 471 -> 297 ms (FP64 pipe 75 -> 89 % busy, 14 % fewer FP64 instructions, 15 % fewer padded
 // entries); N = 210 FACTORISED, 304 trajectories 424 -> 244 ms.
 #include <cuda_runtime.h>
 
