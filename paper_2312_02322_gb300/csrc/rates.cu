@@ -21,7 +21,8 @@
 //       are >= 0, so the cubic is): the integral over every whole piece is linear in the knot values with
 //       weights that depend on the temperature alone (host tables, rate_tables); the piece that u0
 //       cuts (or the ramp) is a quartic times exp(-(U - u0)/kT), i.e. five lower incomplete gamma functions
-//       of integer order; the tail's Gamma(2 + p, U_K/kT) is a Chebyshev series in p per temperature.
+//       of integer order; the tail's Gamma(2 + p, x), x = U_K/kT, is a Chebyshev series in p per temperature
+//       for x >= 0.1 and evaluated for the pair below (kRateChebX).
 //       About 170 FP64 instructions per pair and temperature instead of about 4400: the kernel is bound
 //       by the FP64 pipe, so the instruction count is its time.
 //   quadrature  for every other pair (a value below zero is taken as zero, R3), a u0 at or above U_K, and
@@ -50,6 +51,10 @@ constexpr int kGl = 16;
 constexpr int kRateThreads = 128;          // a block's tile of pairs: 16 levels a x 8 levels b
 constexpr int kRateTa = 16, kRateTb = 8;
 constexpr int kRateCheb = 16;              // Chebyshev coefficients of the tail per temperature
+// The series expands x^-(1+p) Gamma(2+p, x) e^x, which varies over a factor 1/x in p as x = U_K/kT falls: sixteen
+// terms hold the integral to 2e-14 at x = 0.1, 2e-12 at 0.03, 1e-10 at 0.01 and lose every digit by 1e-7.  A
+// temperature with x below this bound evaluates the incomplete gamma function for each pair.
+constexpr double kRateChebX = 0.1;
 
 struct RateArgs {
     double u[kRateMaxK];
@@ -103,6 +108,9 @@ __device__ double upper_gamma_scaled(double s, double x)
     }
     return pow(x, s) * f;
 }
+
+// the closed form's tail factor x^-(1+p) Gamma(2+p, x) e^x for one pair
+__device__ __noinline__ double rate_tail(double p, double x) { return pow(x, -(1.0 + p)) * upper_gamma_scaled(2.0 + p, x); }
 
 // int sigma~ U exp(-(U - u0)/kT) dU by quadrature, piece by piece in increasing U (y, M: the knot values
 // and second derivatives of this thread's pair, `st` doubles apart)
@@ -241,7 +249,7 @@ __global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant
     }
     const double iga = 1.0 / ga, igb = 1.0 / gb;
     // quartic q of the cut piece (or the ramp): sigma~ U = sum_m q_m (U - u0)^m on [u0, U_j]
-    double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0, q4 = 0.0, w = 0.0, chx = 0.0;
+    double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0, q4 = 0.0, w = 0.0, p = 0.0;
     if (closed) {
         w = A.u[j] - u0;
         if (j > 0) {
@@ -261,10 +269,9 @@ __global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant
             q1 = ramp * u0;
             q2 = ramp;
         }
-        // Chebyshev argument 2 p + 1 of the tail's exponent p in [-1, 0]
+        // the tail's exponent
         const double yK = y[(K - 1) * st], yJ = y[(K - 2) * st];
-        chx = 1.0;
-        if (yK > 0.0 && yJ > 0.0) chx = fma(2.0, fmin(0.0, fmax(-1.0, log(yK / yJ) / A.ln_uK)), 1.0);
+        if (yK > 0.0 && yJ > 0.0) p = fmin(0.0, fmax(-1.0, log(yK / yJ) / A.ln_uK));
     }
     for (int t = t0; t < t1; ++t) {
         const double th = A.kT[t], ith = A.ikT[t];
@@ -284,14 +291,20 @@ __global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant
             // left out under the quadrature's remainder bound
             const double eK = ez * __ldg(tab + K * K + j), uK = A.u[K - 1];
             if (!(4.0 * ymax * th * (uK + th) * eK <= 1e-17 * acc)) {
-                const double *ch = tab + K * K + K;
-                double d1 = 0.0, d2 = 0.0;
-                for (int m = kRateCheb - 1; m > 0; --m) {
-                    const double d = fma(2.0 * chx, d1, __ldg(ch + m) - d2);
-                    d2 = d1;
-                    d1 = d;
+                double gp;
+                if (uK * ith >= kRateChebX) {
+                    const double *ch = tab + K * K + K, chx = fma(2.0, p, 1.0);  // [-1, 0] on [-1, 1]
+                    double d1 = 0.0, d2 = 0.0;
+                    for (int m = kRateCheb - 1; m > 0; --m) {
+                        const double d = fma(2.0 * chx, d1, __ldg(ch + m) - d2);
+                        d2 = d1;
+                        d1 = d;
+                    }
+                    gp = fma(chx, d1, __ldg(ch) - d2);
+                } else {
+                    gp = rate_tail(p, uK * ith);
                 }
-                acc = fma(y[(K - 1) * st] * th * uK * eK, fma(chx, d1, __ldg(ch) - d2), acc);
+                acc = fma(y[(K - 1) * st] * th * uK * eK, gp, acc);
             }
         } else {
             acc = rate_quadrature(A, y, M, st, ymax, u0, th, ith);
@@ -452,6 +465,7 @@ void rate_tables(const RateArgs &A, std::vector<double> &tab)
             for (int m = 0; m < K; ++m) W[j * K + m] = row[m];
         }
         // Chebyshev series of g(p) on p in [-1, 0] (s = 2 + p), through its Chebyshev points
+        if (uK / th < 0.5 * kRateChebX) continue;  // not read (half: whatever the rounding of the kernel's ratio)
         double f[kRateCheb];
         for (int i = 0; i < kRateCheb; ++i)
             f[i] = upper_gamma_reduced(1.5 + 0.5 * std::cos(pi * (i + 0.5) / kRateCheb), uK / th);
