@@ -85,7 +85,8 @@ typedef enum { MQCT_FP64 = 0, MQCT_FP32 = 1, MQCT_BF16X3 = 2 } mqct_precision;
 #define MQCT_TRAJ_MAX_STEPS 1   /* max_steps reached before the stop rule (e.g. orbiting)   */
 #define MQCT_TRAJ_TABLE_RANGE 2 /* some stage had R < r_min (end cubic extrapolated)        */
 #define MQCT_TRAJ_NONFINITE 4   /* a non-finite value appeared; the trajectory was stopped  */
-#define MQCT_TRAJ_TIMEOUT 8     /* a bounded device wait ran out while running it           */
+#define MQCT_TRAJ_TIMEOUT 8     /* a bounded device wait ran out while running it: its      */
+                                /* populations and amplitudes are NaN                       */
 #define MQCT_TRAJ_INVALID 16    /* device-resident trajectory failed validation; not run    */
 #define MQCT_TRAJ_CKPT 32       /* adjoint: the forward pass outran its checkpoint storage  */
 
@@ -330,8 +331,8 @@ mqct_status mqct_system_info(mqct_system sys, mqct_system_info_t *out);
  * whether trajectories are still running), and BF16X3 calls with several systems synchronise
  * it once to size the per-system launches.  With any host
  * output the call synchronises the stream and returns MQCT_ERR_TRAJ if a trajectory status
- * is non-zero.  Errors: MQCT_ERR_INVALID_ARG, MQCT_ERR_UNSUPPORTED, MQCT_ERR_OOM,
- * MQCT_ERR_CUDA, MQCT_ERR_TRAJ. */
+ * is non-zero (MQCT_ERR_TIMEOUT if one has MQCT_TRAJ_TIMEOUT).  Errors: MQCT_ERR_INVALID_ARG,
+ * MQCT_ERR_UNSUPPORTED, MQCT_ERR_OOM, MQCT_ERR_CUDA, MQCT_ERR_TIMEOUT, MQCT_ERR_TRAJ. */
 mqct_status mqct_propagate(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs, int32_t n,
                            double *final_pop, double *final_amp, mqct_diag *diag, void *cuda_stream);
 

@@ -1,5 +1,5 @@
 /*
- * mqct_probe.h -- arithmetic-throughput probes of the GPU the library runs on.
+ * mqct_probe.h -- probes of the GPU the library runs on and checks of the library's building blocks.
  *
  * Not part of the paper's method: the roofline of the FP64 trajectory kernels is the
  * FP64 fused-multiply-add rate, which the measured-peaks file of the machine does not
@@ -37,6 +37,15 @@ mqct_status mqct_probe_op_latency(int32_t kind, int32_t warps, double *cycles, v
  * Errors: MQCT_ERR_INVALID_ARG, MQCT_ERR_TIMEOUT (the bounded completion wait ran out),
  * MQCT_ERR_CUDA.  No counterpart in the paper (a building-block check). */
 mqct_status mqct_probe_tc_gemm(int32_t n, int32_t k, const void *a, const void *b, float *d, void *cuda_stream);
+
+/* mqct_propagate_ex in which bounded device waits run out (a check of that path without a hang): in the FP32 batched
+ * kernel a thread block that claims work item fail_every - 1, 2 fail_every - 1, ... of a system's work list
+ * (fail_every > 0) behaves as if one of its waits had then run out.  The trajectories that it holds get status
+ * MQCT_TRAJ_TIMEOUT and NaN results when they end, and the block goes on with the next ones.  Other kernels ignore it.
+ * Errors: as mqct_propagate_ex, plus MQCT_ERR_INVALID_ARG for fail_every < 0. */
+mqct_status mqct_probe_propagate_timeout(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs, int32_t n,
+                                         double *final_pop, double *final_amp, mqct_diag *diag,
+                                         const mqct_propagate_opts *opts, int32_t fail_every, void *cuda_stream);
 
 #ifdef __cplusplus
 }

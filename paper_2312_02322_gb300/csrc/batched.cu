@@ -181,7 +181,9 @@ struct BatchShared {
     SlotCold cold[B];
     int live[B > 8 ? B / 8 : 1];  // per slot warp: some slot of it is not idle (set at stage 0)
     int cur;                      // system the CTA is bound to (-1: no work left)
-    int timeout;                  // a bounded wait ran out
+    // a bounded wait of an element warp ran out (since the CTA bound to this system): what the slots hold is void,
+    // the CTA claims nothing more and binds anew once they have ended
+    int timeout;
     __align__(8) uint64_t published;  // mbarrier: the slot warps have published a stage's views
 };
 
@@ -230,6 +232,16 @@ __device__ int pick_system(const BatchMultiArgs &a, bool first)
         }
     }
     return best;
+}
+
+// the results of a trajectory that a timeout made void (row offset o): NaN; by four lanes, this one the c-th
+__device__ __noinline__ void batched_void(double *pop, double *amp, size_t o, int n, int c)
+{
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    for (int r = c; r < n; r += 4) {
+        if (pop) pop[o + r] = nan;
+        if (amp) amp[2 * (o + r)] = amp[2 * (o + r) + 1] = nan;
+    }
 }
 
 // everything a CTA does while bound to system `cur`: with BC > 0 its slot count is the compile-time
@@ -315,13 +327,14 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
     // on return the slot is WAIT (column to be initialised at the next stage 3) or IDLE
     auto claim = [&]() {
         for (;;) {
-            int item = 0;
-            if (sc == 0) item = atomicAdd(queue, 1);
+            int item = count;
+            if (sc == 0 && !sh.timeout) item = atomicAdd(queue, 1);
             item = __shfl_sync(m4, item, sj);
             if (item >= count) {
                 state = SLOT_IDLE;
                 return;
             }
+            if (a.fail_every && sc == 0 && (item + 1) % a.fail_every == 0) sh.timeout = 1;
             const int t = order ? order[item] : item;
             const mqct_traj tr = a.trajs[t];
             if (!traj_valid(tr, S, a.sys_base + cur)) {
@@ -549,7 +562,10 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
             }
             __syncwarp();
             if (lane == 0) tc_mbar_arrive(&sh.published);
-            if (!run) break;
+            if (!run) {  // the element warps read `live` after the barrier
+                __syncthreads();
+                break;
+            }
             // ---- bookkeeping of stage 0 (a finished slot at stage 1, before its refill; running slots
             // at stage 2), the diagnostics and refill of a finished slot, then the look-ahead
             if (s == 1) {
@@ -558,10 +574,12 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
                 if (fin_any) {
                     bookkeeping(slot_lane && state == SLOT_FINAL);
                     if (slot_lane && state == SLOT_FINAL) {
+                        const int out = __shfl_sync(m4, sh.timeout, sj);
+                        if (out) batched_void(a.pop, a.amp, (size_t)cs.traj * a.nmax, n, sc);
                         if (sc == 0) {
                             if (a.diag) {
                                 mqct_diag d;
-                                d.steps = steps; d.status = cs.status | (sh.timeout ? MQCT_TRAJ_TIMEOUT : 0);
+                                d.steps = steps; d.status = cs.status | (out ? MQCT_TRAJ_TIMEOUT : 0);
                                 d.norm_dev = cs.ndev; d.energy_dev = cs.edev; d.angmom_dev = cs.jdev;
                                 d.t_final = steps * dtd;
                                 a.diag[cs.traj] = d;
@@ -623,8 +641,8 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
     }
     __syncthreads();
 
-    // one RK4 stage of this warp's units; false once no slot is live
-    auto stage = [&](auto s0c, int s) -> bool {
+    // one RK4 stage of this warp's units
+    auto stage = [&](auto s0c, int s) {
         constexpr bool S0 = decltype(s0c)::value;
         const int par = s & 1;
         const SlotView<BMAX> &vw = sh.view[par];
@@ -636,7 +654,8 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
         // the views of this stage, which the slot warps publish during the contraction: every lane of the
         // warp waits, and the warp converges again afterwards
         auto wait = [&]() {
-            // (bounded; after one wait ran out the others return at once and the results carry the flag)
+            // (bounded; after one wait ran out the others return at once: the stages go on with whatever the views
+            // hold, whose indices are in range at any time, and the results are void)
             if (!*(volatile int *)&sh.timeout && !tc_mbar_wait(&sh.published, phase & 1u, kBatchWait)) sh.timeout = 1;
             __syncwarp();
             const int4 st4 = *reinterpret_cast<const int4 *>(vw.state + 4 * g);
@@ -838,12 +857,6 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
         }
         __syncwarp();
         ++phase;
-        if (S0) {
-            bool run = false;
-#pragma unroll
-            for (int i = 0; i < NS; ++i) run |= sh.live[i] != 0;
-            if (!run) return false;
-        }
         // phase factors of the stages ahead: t + dt once stage 0 has read those of t, the next step's half
         // time once stage 2 has read this one's (t = 0 of a starting slot needs none)
         if (!S0 && s != 2) {
@@ -908,11 +921,15 @@ __device__ __forceinline__ void batched_system(const BatchMultiArgs &a, BatchSha
         }
         any = act;
         __syncwarp();
-        return true;
     };
     for (;;) {
-        if (!stage(std::true_type{}, 0)) break;
+        stage(std::true_type{}, 0);
         __syncthreads();
+        // (read behind the barrier: whether or not a wait ran out, both roles leave at the same stage)
+        bool run = false;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) run |= sh.live[i] != 0;
+        if (!run) break;
 #pragma unroll 1
         for (int s = 1; s < 4; ++s) {
             stage(std::false_type{}, s);
@@ -933,15 +950,13 @@ __global__ void __launch_bounds__(T, batched_min_blocks<T>()) k_batched_f32(Batc
     __shared__ BatchShared<BMAX> sh;
     bool first = true;
     unsigned phase = 0;  // stages published so far (parity of the mbarrier)
-    if (threadIdx.x == 0) {
-        sh.timeout = 0;
-        tc_mbar_init(&sh.published, batch_slot_warps(BMAX));
-    }
+    if (threadIdx.x == 0) tc_mbar_init(&sh.published, batch_slot_warps(BMAX));
     for (;;) {
         // bind to a system
         if (threadIdx.x == 0) {
             const int s = pick_system(a, first);
             sh.cur = s;
+            sh.timeout = 0;
             if (s >= 0) sh.S = a.sys[s];
         }
         __syncthreads();

@@ -157,6 +157,7 @@ struct BatchMultiArgs {
     mqct_diag *diag;
     long long *t_start, *t_done;  // optional device clock (ns) at start / end of each trajectory
     int nmax;
+    int fail_every;               // mqct_probe_propagate_timeout; 0: none
 };
 // the (slots per CTA at most, threads) instances of the FP32 batched kernel; batched_auto_shape
 // picks one from the trajectory count and the slots each shape gives the systems

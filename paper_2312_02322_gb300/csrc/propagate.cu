@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "mqct_probe.h"
 #include "tc_ptx.cuh"
 #include "traj_common.cuh"
 
@@ -745,9 +746,10 @@ extern "C" mqct_status mqct_propagate(const mqct_system *systems, int32_t n_syst
     return mqct_propagate_ex(systems, n_systems, trajs, n, final_pop, final_amp, diag, nullptr, cuda_stream);
 }
 
-extern "C" mqct_status mqct_propagate_ex(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs,
-                                         int32_t n, double *final_pop, double *final_amp, mqct_diag *diag,
-                                         const mqct_propagate_opts *opts, void *cuda_stream)
+// mqct_propagate_ex; fail_every as in mqct_probe_propagate_timeout
+static mqct_status propagate_impl(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs, int32_t n,
+                                  double *final_pop, double *final_amp, mqct_diag *diag,
+                                  const mqct_propagate_opts *opts, int fail_every, void *cuda_stream)
 {
     reset_launches();
     const mqct_propagate_opts no_opts{};
@@ -881,7 +883,7 @@ extern "C" mqct_status mqct_propagate_ex(const mqct_system *systems, int32_t n_s
             // launch): CTAs bind to systems on the device
             BatchMultiArgs ma{};
             ma.trajs = dtr; ma.pop = dpop; ma.amp = damp; ma.diag = ddiag; ma.nmax = nmax;
-            ma.t_start = dts; ma.t_done = dtd; ma.n = n;
+            ma.t_start = dts; ma.t_done = dtd; ma.n = n; ma.fail_every = fail_every;
             int shape = 0;
             for (int i = 0; i < n_systems && !shape; ++i) shape = shape_of(i);
             for (int g0 = 0; g0 < n_systems; g0 += kBatchMaxSystems) {
@@ -949,7 +951,24 @@ extern "C" mqct_status mqct_propagate_ex(const mqct_system *systems, int32_t n_s
     if ((e = cudaMemcpyAsync(dst, ddiag, sizeof(mqct_diag) * (size_t)n, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
         return cuda_fail(e, "cudaMemcpyAsync");
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    for (int i = 0; i < n; ++i)
-        if (dst[i].status != 0) return fail(MQCT_ERR_TRAJ, "at least one trajectory ended with a non-zero status");
+    int all = 0;
+    for (int i = 0; i < n; ++i) all |= dst[i].status;
+    if (all & MQCT_TRAJ_TIMEOUT) return fail(MQCT_ERR_TIMEOUT, "mqct_propagate: a bounded device wait ran out");
+    if (all) return fail(MQCT_ERR_TRAJ, "at least one trajectory ended with a non-zero status");
     return MQCT_OK;
+}
+
+extern "C" mqct_status mqct_propagate_ex(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs,
+                                         int32_t n, double *final_pop, double *final_amp, mqct_diag *diag,
+                                         const mqct_propagate_opts *opts, void *cuda_stream)
+{
+    return propagate_impl(systems, n_systems, trajs, n, final_pop, final_amp, diag, opts, 0, cuda_stream);
+}
+
+extern "C" mqct_status mqct_probe_propagate_timeout(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs,
+                                                    int32_t n, double *final_pop, double *final_amp, mqct_diag *diag,
+                                                    const mqct_propagate_opts *opts, int32_t fail_every, void *cuda_stream)
+{
+    if (fail_every < 0) return fail(MQCT_ERR_INVALID_ARG, "mqct_probe_propagate_timeout: fail_every < 0");
+    return propagate_impl(systems, n_systems, trajs, n, final_pop, final_amp, diag, opts, fail_every, cuda_stream);
 }
