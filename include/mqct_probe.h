@@ -38,10 +38,11 @@ mqct_status mqct_probe_op_latency(int32_t kind, int32_t warps, double *cycles, v
  * MQCT_ERR_CUDA.  No counterpart in the paper (a building-block check). */
 mqct_status mqct_probe_tc_gemm(int32_t n, int32_t k, const void *a, const void *b, float *d, void *cuda_stream);
 
-/* mqct_propagate_ex in which bounded device waits run out (a check of that path without a hang): in the FP32 batched
- * kernel a thread block that claims work item fail_every - 1, 2 fail_every - 1, ... of a system's work list
- * (fail_every > 0) behaves as if one of its waits had then run out.  The trajectories that it holds get status
- * MQCT_TRAJ_TIMEOUT and NaN results when they end, and the block goes on with the next ones.  Other kernels ignore it.
+/* mqct_propagate_ex in which bounded device waits run out (a check of that path without a hang): in the FP64 and the
+ * FP32 batched kernels a thread block that claims work item fail_every - 1, 2 fail_every - 1, ... of the work list
+ * (FP32: of a system's; fail_every > 0) behaves as if one of its waits had then run out.  The trajectories that it
+ * holds get status MQCT_TRAJ_TIMEOUT and NaN results when they end, and the block goes on with the next ones.  The
+ * stage-synchronous paths ignore it.
  * Errors: as mqct_propagate_ex, plus MQCT_ERR_INVALID_ARG for fail_every < 0. */
 mqct_status mqct_probe_propagate_timeout(const mqct_system *systems, int32_t n_systems, const mqct_traj *trajs, int32_t n,
                                          double *final_pop, double *final_amp, mqct_diag *diag,

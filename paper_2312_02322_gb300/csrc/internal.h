@@ -110,6 +110,7 @@ struct PropArgs {
     int smem_n;    // shared-memory vector length (max n over systems)
     int smem_lev;  // max n_levels over systems
     int adapt;     // some system uses adaptive steps: two more vectors of smem_n in shared memory
+    int fail_every;  // mqct_probe_propagate_timeout; 0: none
 };
 // launches it over pa.n trajectories; pa.nmax: the largest basis, maxlev: the most levels, adapt: some system
 // uses adaptive steps.  cudaErrorInvalidConfiguration: it does not fit on an SM

@@ -59,7 +59,8 @@ struct Ctl {
     double err, tcur;
     double red[kPropElem][6];            // sums of one stage per element warp
     int kint[2];
-    int below_n, status, steps, done, max_steps, item, timeout;
+    int below_n, status, steps, done, max_steps, item;
+    int timeout;                         // a bounded wait ran out: the trajectory's results are void
     __align__(8) uint64_t published;     // mbarrier: classical and phase warp are done with what a stage needs
 };
 
@@ -285,7 +286,8 @@ __device__ __forceinline__ void elem_stage(const DevSys &S, Ctl &c, int s, int n
     const double2 *PHc = (S0 || s == 3) ? PHa : PHb, *PHn = (S0 || s == 1) ? PHb : PHa;
     const double hb = (!S0 && s == 3) ? c.h6 : (s == 2 ? c.h : c.hh);
     double f = 0.0, t = 0.0, ve = 0.0, jy = 0.0, nr = 0.0, er = 0.0;
-    // every lane of the warp waits for the views of this stage, and the warp converges again afterwards
+    // every lane of the warp waits for the views of this stage, and the warp converges again afterwards (bounded;
+    // after one wait ran out the trajectory's others return at once)
     auto wait = [&]() {
         if (!*(volatile int *)&c.timeout && !tc_mbar_wait(&c.published, phase & 1u, kPropWait)) c.timeout = 1;
         __syncwarp();
@@ -371,10 +373,7 @@ __global__ void __launch_bounds__(T, MINB) k_propagate_fp64(PropArgs a)
     double *Ad = reinterpret_cast<double *>(A), *ACCd = reinterpret_cast<double *>(ACC);
     double *C0d = reinterpret_cast<double *>(C0), *C1d = reinterpret_cast<double *>(C1);
     unsigned phase = 0;  // stages published so far (parity of the mbarrier)
-    if (tid == 0) {
-        c.timeout = 0;
-        tc_mbar_init(&c.published, 2);
-    }
+    if (tid == 0) tc_mbar_init(&c.published, 2);
 
     for (;;) {
         if (tid == 0) c.item = atomicAdd(a.queue, 1);
@@ -397,6 +396,7 @@ __global__ void __launch_bounds__(T, MINB) k_propagate_fp64(PropArgs a)
         }
         if (tid == 0) {
             S = a.sys[tr.system_idx];
+            c.timeout = a.fail_every > 0 && (item + 1) % a.fail_every == 0;
             if (a.t_start) a.t_start[t] = mqct_clock_ns();
         }
         __syncthreads();
@@ -598,6 +598,7 @@ __global__ void __launch_bounds__(T, MINB) k_propagate_fp64(PropArgs a)
             }
         }
         // ---- diagnostics of the final state
+        const bool out = c.timeout;
         if (classical) {
             if (!(c.status & MQCT_TRAJ_NONFINITE)) {
                 if (lane == 0) { c.i2m0 = c.i2m; c.vid0 = c.vid[0]; }
@@ -607,7 +608,7 @@ __global__ void __launch_bounds__(T, MINB) k_propagate_fp64(PropArgs a)
             if (lane == 0) {
                 if (a.diag) {
                     mqct_diag d;
-                    d.steps = c.steps; d.status = c.status | (c.timeout ? MQCT_TRAJ_TIMEOUT : 0);
+                    d.steps = c.steps; d.status = c.status | (out ? MQCT_TRAJ_TIMEOUT : 0);
                     d.norm_dev = c.ndev; d.energy_dev = c.edev; d.angmom_dev = c.jdev;
                     d.t_final = c.tcur;
                     a.diag[t] = d;
@@ -615,7 +616,12 @@ __global__ void __launch_bounds__(T, MINB) k_propagate_fp64(PropArgs a)
                 if (a.t_done) a.t_done[t] = mqct_clock_ns();
             }
         }
-        // ---- outputs in the caller's state order
+        // ---- outputs in the caller's state order (NaN after a timeout)
+        if (elem && out)
+            for (int r = tid; r < n; r += nte) {
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                A[r] = make_double2(nan, nan);
+            }
         if (elem) {
             if (a.pop)
                 for (int r = tid; r < n; r += nte) {
@@ -925,7 +931,7 @@ static mqct_status propagate_impl(const mqct_system *systems, int32_t n_systems,
     PropArgs pa{};
     pa.sys = dsys; pa.trajs = dtr; pa.order = order; pa.n = n; pa.n_systems = n_systems; pa.queue = queue;
     pa.pop = dpop; pa.amp = damp; pa.diag = ddiag; pa.nmax = nmax;
-    pa.t_start = dts; pa.t_done = dtd;
+    pa.t_start = dts; pa.t_done = dtd; pa.fail_every = fail_every;
     if ((e = launch_propagate(pa, maxlev, adapt, st)) != cudaSuccess) {
         if (e == cudaErrorInvalidConfiguration) return fail(MQCT_ERR_UNSUPPORTED, "mqct_propagate: kernel does not fit on an SM");
         return cuda_fail(e, "k_propagate_fp64 launch (basis too large for shared memory?)");

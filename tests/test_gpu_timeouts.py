@@ -98,3 +98,25 @@ def test_fp32_without_diagnostics():
     assert st == 0 and np.all(np.isfinite(pop))
     # host outputs and no diagnostics: the status of the call
     assert _call(s, tr, 1, diag=False)[0] == ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("path", ["plain", "factorised"])
+@pytest.mark.parametrize("adapt", [None, (1e-6, 4)])
+@pytest.mark.parametrize("jmax,n", [(2, 1000), (13, 200)])
+def test_fp64_trajectory_alone_is_void(path, adapt, jmax, n):
+    import paper_2312_02322_gb300.api as mq
+
+    s = mq.System.diatom(W.diatom_pes_params(jmax=jmax, n_grid=120), path=path, precision="fp64", adapt=adapt)
+    tr = _trajs(mq, n, 20, 7)
+    for fail_every in (0, 1, 3, n, n + 1):
+        assert _check(mq, s, tr, fail_every).sum() == (n // fail_every if fail_every else 0)
+
+
+def test_fp64_without_diagnostics():
+    import paper_2312_02322_gb300.api as mq
+
+    s = mq.System.diatom(W.diatom_pes_params(jmax=3, n_grid=120), path="plain", precision="fp64")
+    tr = _trajs(mq, 9, 20, 6)
+    st, pop, _, _ = _call(s, tr, 2, device=True)
+    assert st == 0 and np.all(np.isnan(pop), axis=1).sum() == 4 and np.isnan(pop).sum() == 4 * s.n
+    assert _call(s, tr, 2, diag=False)[0] == ERR_TIMEOUT
