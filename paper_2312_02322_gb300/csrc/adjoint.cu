@@ -938,6 +938,9 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         if (t.system_idx != 0 || t.init_state < 0 || t.init_state >= h.n || !(t.dt > 0) || !(t.e_coll > 0) ||
             !(t.b >= 0) || !(t.r0 > t.b) || t.max_steps < 0 || !std::isfinite(t.r_end))
             return fail(MQCT_ERR_INVALID_ARG, "mqct_adjoint: invalid trajectory");
+        // as mqct_propagate: a start inside the centrifugal barrier, an energy that overflows
+        const double q = 2.0 * h.mu * t.e_coll - 2.0 * h.mu * t.e_coll * (t.b * t.b) / (t.r0 * t.r0);
+        if (!(q > 0)) return fail(MQCT_ERR_INVALID_ARG, "mqct_adjoint: trajectory starts inside its centrifugal barrier (b >= r0)");
     }
     // what the forward propagation refuses, the adjoint refuses (one trajectory of no steps)
     {
