@@ -48,6 +48,13 @@ mqct_status mqct_probe_propagate_timeout(const mqct_system *systems, int32_t n_s
                                          double *final_pop, double *final_amp, mqct_diag *diag,
                                          const mqct_propagate_opts *opts, int32_t fail_every, void *cuda_stream);
 
+/* mqct_adjoint on a device where no allocation of its checkpoints and work vectors above `limit` bytes succeeds (a
+ * check of what it does when it is short of memory).
+ * Errors: as mqct_adjoint, plus MQCT_ERR_INVALID_ARG for limit < 0. */
+mqct_status mqct_probe_adjoint_limit(mqct_system sys, const mqct_traj *trajs, int32_t n, const double *weight,
+                                     const int32_t *group, int32_t n_groups, const double *dL_dsigma, int32_t ckpt,
+                                     double *dL_dparam, int64_t limit, void *cuda_stream);
+
 #ifdef __cplusplus
 }
 #endif

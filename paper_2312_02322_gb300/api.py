@@ -143,6 +143,8 @@ def lib():
             L.mqct_probe_op_latency.restype = C.c_int
             L.mqct_probe_propagate_timeout.argtypes = [C.POINTER(vp), i32, vp, i32, vp, vp, vp, C.POINTER(PropagateOpts), i32, vp]
             L.mqct_probe_propagate_timeout.restype = C.c_int
+            L.mqct_probe_adjoint_limit.argtypes = [vp, vp, i32, vp, vp, i32, vp, i32, vp, i64, vp]
+            L.mqct_probe_adjoint_limit.restype = C.c_int
             L.mqct_last_error.restype = C.c_char_p
             L.mqct_last_launch_count.restype = C.c_int64
             L.mqct_version.restype = C.c_char_p

@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "mqct_probe.h"
 #include "traj_common.cuh"
 
 namespace mqct {
@@ -895,9 +896,10 @@ bool adj_is_dev(const void *p)
 }
 }  // namespace
 
-extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int32_t n, const double *weight,
-                                    const int32_t *group, int32_t n_groups, const double *dL_dsigma, int32_t ckpt,
-                                    double *dL_dparam, void *cuda_stream)
+// mqct_adjoint; an allocation of checkpoints and work vectors above `limit` bytes counts as one that failed
+static mqct_status adjoint_impl(mqct_system sys, const mqct_traj *trajs, int32_t n, const double *weight,
+                                const int32_t *group, int32_t n_groups, const double *dL_dsigma, int32_t ckpt,
+                                double *dL_dparam, size_t limit, void *cuda_stream)
 {
     reset_launches();
     if (sys && sys->s.h.grid_log) return fail(MQCT_ERR_UNSUPPORTED, "mqct_adjoint: the logarithmic grid is not supported");
@@ -964,7 +966,7 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     const size_t stride = amp_bytes + 32;
     // a recomputed step keeps its three later stage states and the classical stage states too: the reverse
     // sweep then needs no second recomputation (a fifth of a gradient); left out when the segments of all
-    // CTAs would take more than 16 GB
+    // CTAs would take more than 16 GB or the allocation fails
     const size_t stage_bytes = ((6 * (size_t)h.n * rsz + 15) & ~(size_t)15) + 16 * sizeof(double);
     // work vectors: 17 of length N and the phase factors of every level, in shared memory when
     // they fit, else in a global-memory region per CTA
@@ -984,7 +986,7 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         return cuda_fail(e, "cudaFuncSetAttribute");
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, smem)) != cudaSuccess)
         return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    const int grid = std::max(1, std::min(n, sms * std::max(per_sm, 1)));
+    int grid = std::max(1, std::min(n, sms * std::max(per_sm, 1)));
     auto count_steps = [&](int &steps) -> mqct_status {
         std::vector<mqct_diag> dg(n);
         mqct_system one = sys;
@@ -1002,8 +1004,6 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
     } else {
         max_steps = (int)bound;
     }
-    const bool stages = (size_t)grid * ckpt * (stride + stage_bytes) <= (size_t)16 << 30;
-    const size_t seg_stride = stride + (stages ? stage_bytes : 0);
     std::vector<void *> tmp;
     auto get = [&](void **p, size_t b) {
         cudaError_t r = cudaMallocAsync(p, b ? b : 16, st);
@@ -1034,14 +1034,11 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         return cuda_fail(e, "staging");
     }
     aa.dLds = (const double *)ptr;
-    aa.n = n; aa.n_groups = n_groups; aa.K = ckpt; aa.stride = stride;
-    aa.seg_stride = seg_stride; aa.stages = stages ? 1 : 0;
+    aa.n = n; aa.n_groups = n_groups; aa.stride = stride;
     int *queue = nullptr;
-    unsigned char *vec = nullptr;
     double *theta = nullptr, *out = nullptr;
     int *status = nullptr;
     if ((e = get((void **)&queue, sizeof(int))) != cudaSuccess ||
-        (vec_global && (e = get((void **)&vec, (size_t)grid * vec_bytes)) != cudaSuccess) ||
         (e = get((void **)&theta, sizeof(double) * (size_t)n * h.P)) != cudaSuccess ||
         (e = get((void **)&status, sizeof(int) * (size_t)n)) != cudaSuccess ||
         (e = get((void **)&out, sizeof(double) * h.P)) != cudaSuccess) {
@@ -1049,18 +1046,25 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         return cuda_fail(e, "cudaMallocAsync (adjoint scratch)");
     }
     aa.queue = queue; aa.theta_traj = theta; aa.status = status;
-    aa.vec = vec; aa.vec_bytes = vec_bytes;
+    aa.vec_bytes = vec_bytes;
     std::vector<int> hst(n);
     int launches = 0;
+    bool short_of_memory = false;
     for (;;) {
-        aa.max_ckpt = max_steps / ckpt + 2;
+        // an interval longer than the trajectories needs no storage beyond their steps
+        aa.K = std::min(ckpt, std::max(1, max_steps));
+        aa.max_ckpt = max_steps / aa.K + 2;
+        aa.stages = !short_of_memory && (size_t)grid * aa.K * (stride + stage_bytes) <= (size_t)16 << 30;
+        aa.seg_stride = stride + (aa.stages ? stage_bytes : 0);
+        const size_t vec_all = vec_global ? (size_t)grid * vec_bytes : 0;
+        const size_t need = vec_all + (size_t)grid * ((size_t)aa.max_ckpt * stride + (size_t)aa.K * aa.seg_stride);
         void *scratch = nullptr;
-        e = cudaMallocAsync(&scratch, (size_t)grid * ((size_t)aa.max_ckpt * stride + (size_t)ckpt * aa.seg_stride), st);
-        if (e == cudaErrorMemoryAllocation && (aa.stages || !counted)) {
-            // short of memory: the least that the call can do with, no stage states and counted steps
+        e = need > limit ? cudaErrorMemoryAllocation : cudaMallocAsync(&scratch, need, st);
+        if (e == cudaErrorMemoryAllocation && (aa.stages || !counted || grid > sms)) {
+            // short of memory: no stage states and counted steps, then one CTA per SM
             cudaGetLastError();
-            aa.stages = 0;
-            aa.seg_stride = stride;
+            if (!aa.stages && counted) grid = sms;
+            short_of_memory = true;
             if (!counted) {
                 const mqct_status s2 = count_steps(max_steps);
                 if (s2 != MQCT_OK) { cleanup(); return s2; }
@@ -1072,7 +1076,8 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
             cleanup();
             return cuda_fail(e, "cudaMallocAsync (adjoint checkpoints)");
         }
-        aa.scratch = static_cast<unsigned char *>(scratch);
+        aa.vec = vec_global ? static_cast<unsigned char *>(scratch) : nullptr;
+        aa.scratch = static_cast<unsigned char *>(scratch) + vec_all;
         cudaMemsetAsync(queue, 0, sizeof(int), st);
         if (fp32) k_adjoint<float><<<grid, kAdjThreads, smem, st>>>(aa);
         else k_adjoint<double><<<grid, kAdjThreads, smem, st>>>(aa);
@@ -1101,4 +1106,19 @@ extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int
         if (hst[i] != 0 && hst[i] != MQCT_TRAJ_TABLE_RANGE)
             return fail(MQCT_ERR_TRAJ, "mqct_adjoint: a trajectory did not end normally (excluded from the gradient)");
     return MQCT_OK;
+}
+
+extern "C" mqct_status mqct_adjoint(mqct_system sys, const mqct_traj *trajs, int32_t n, const double *weight,
+                                    const int32_t *group, int32_t n_groups, const double *dL_dsigma, int32_t ckpt,
+                                    double *dL_dparam, void *cuda_stream)
+{
+    return adjoint_impl(sys, trajs, n, weight, group, n_groups, dL_dsigma, ckpt, dL_dparam, SIZE_MAX, cuda_stream);
+}
+
+extern "C" mqct_status mqct_probe_adjoint_limit(mqct_system sys, const mqct_traj *trajs, int32_t n, const double *weight,
+                                                const int32_t *group, int32_t n_groups, const double *dL_dsigma, int32_t ckpt,
+                                                double *dL_dparam, int64_t limit, void *cuda_stream)
+{
+    if (limit < 0) return fail(MQCT_ERR_INVALID_ARG, "mqct_probe_adjoint_limit: limit < 0");
+    return adjoint_impl(sys, trajs, n, weight, group, n_groups, dL_dsigma, ckpt, dL_dparam, (size_t)limit, cuda_stream);
 }
