@@ -953,13 +953,14 @@ static mqct_status adjoint_impl(mqct_system sys, const mqct_traj *trajs, int32_t
         const mqct_status s2 = mqct_propagate(&one, 1, &t0, 1, nullptr, nullptr, &d0, cuda_stream);
         if (s2 != MQCT_OK && s2 != MQCT_ERR_TRAJ) return s2;
     }
-    // Checkpoint storage: three free flights 2 r0 / v of every trajectory, at most its max_steps.  A trajectory
-    // that outruns it (an orbiting one; status CKPT) makes the call count the steps by a forward propagation and
+    // Checkpoint storage: three free flights from r0 to the centre and out to r_end (at least r0) of every
+    // trajectory, at most its max_steps.  A trajectory that outruns it (an orbiting one; status CKPT) makes the call count the steps by a forward propagation and
     // run again; so does storage above 4 GB, before the first run.  N = 441, against a counting propagation in
     // every call: FP64, 128 trajectories, 695 -> 601 ms; mixed, 256 trajectories, 313 -> 286.
     double bound = 1.0;
     for (const mqct_traj &t : ht)
-        bound = std::max(bound, std::min((double)t.max_steps, 64.0 + 6.0 * t.r0 / (t.dt * std::sqrt(2.0 * t.e_coll / h.mu))));
+        bound = std::max(bound, std::min((double)t.max_steps,
+                                         64.0 + 3.0 * (t.r0 + std::max(t.r0, t.r_end)) / (t.dt * std::sqrt(2.0 * t.e_coll / h.mu))));
     // a stored state: amplitudes (FP32: and their compensation terms), then 4 classical doubles
     const size_t rsz = fp32 ? sizeof(float) : sizeof(double);
     const size_t amp_bytes = ((fp32 ? 4 : 2) * (size_t)h.n * rsz + 15) & ~(size_t)15;
