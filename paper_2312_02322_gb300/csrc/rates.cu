@@ -50,6 +50,7 @@ constexpr int kRateMaxT = MQCT_RATE_MAX_TEMPS;
 constexpr int kGl = 16;
 constexpr int kRateThreads = 128;          // a block's tile of pairs: 16 levels a x 8 levels b
 constexpr int kRateTa = 16, kRateTb = 8;
+constexpr size_t kRatePass = (size_t)1 << 26;  // pairs of levels of one pass (all up to 11 585 levels): 512 MB of list
 constexpr int kRateCheb = 16;              // Chebyshev coefficients of the tail per temperature
 // The series expands x^-(1+p) Gamma(2+p, x) e^x, which varies over a factor 1/x in p as x = U_K/kT falls: sixteen
 // terms hold the integral to 2e-14 at x = 0.1, 2e-12 at 0.03, 1e-10 at 0.01 and lose every digit by 1e-7.  A
@@ -70,6 +71,12 @@ struct RateArgs {
     // per temperature: [K][K] weights of the whole pieces at and above knot j, [K] exp(-(U_K - U_j)/kT),
     // the tail's Chebyshev coefficients
     const double *tab;
+};
+
+// the pairs whose rates k_rates leaves to k_rates_quad, listed from the front (whole warps of them, which stay
+// together: their panel counts are alike) and from the back (the others); the next item of k_rates_quad
+struct RateQueue {
+    unsigned long long front, back, next, pad;
 };
 
 // doubles of A.tab per temperature
@@ -203,17 +210,28 @@ __device__ __forceinline__ void lower_gammas(double z, double ez, double G[5])
     }
 }
 
-// One thread per unordered pair (a <= b): the symmetrised cross sections of Eq. 20 (out, or NULL) and
-// both rates.  A block takes a tile of 16 x 8 pairs, so that the transposed reads sigma[k][a][b] of its
-// warps share 32-byte sectors.  Bound by the FP64 pipe: 1032 levels x 10 energies x 5 temperatures, all in
-// closed form, take 0.94 ms; the quadrature of every pair took 28.0 ms (one thread per pair and
-// temperature, a separate launch for the symmetrised cross sections).
+// both rates of a pair from its integral (x0 = u0/kT): exp(-dE/(2kT)) exp(-u0/kT) is exp(-|dE|/kT) for an
+// excitation, 1 for a quenching
+__device__ __forceinline__ void rate_store(const RateArgs &A, double *rate, int t, double acc, double dE, double x0,
+                                           double ga, double gb, int ia, int ib)
+{
+    const double c = A.pref[t] * acc, ex = exp(-2.0 * x0);
+    rate[(size_t)ia * A.L + ib] = c * (dE >= 0.0 ? ex : 1.0) * (1.0 / ga);
+    rate[(size_t)ib * A.L + ia] = c * (dE >= 0.0 ? 1.0 : ex) * (1.0 / gb);
+}
+
+// One thread per unordered pair (a <= b): the symmetrised cross sections of Eq. 20 (sym, or NULL) and, where the
+// closed form holds, both rates; the other pairs join the list that k_rates_quad integrates, so that no thread waits
+// for a quadrature.  A block takes a tile of 16 x 8 pairs (rows from b_first on), so that the transposed reads
+// sigma[k][a][b] of its warps share 32-byte sectors.  Bound by the FP64 pipe: a call with 1032 levels x 10 energies x
+// 5 temperatures, all in closed form, takes 1.26 ms (the kernel 0.94); with the quadrature of every pair 27 ms.
 __global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant__ RateArgs A, const double *sigma,
-                                                         const double *g, const double *E, double *sym, double *rate)
+                                                         const double *g, const double *E, double *sym, double *rate,
+                                                         int b_first, RateQueue *queue, int2 *list, size_t list_n)
 {
     extern __shared__ double rsm[];
     const int K = A.K, L = A.L;
-    const int a0 = blockIdx.x * kRateTa, b0 = blockIdx.y * kRateTb;
+    const int a0 = blockIdx.x * kRateTa, b0 = b_first + blockIdx.y * kRateTb;
     if (a0 > b0 + kRateTb - 1) return;
     const int ia = a0 + threadIdx.x % kRateTa, ib = b0 + threadIdx.x / kRateTa;
     if (ia >= L || ib >= L || ia > ib) return;
@@ -247,73 +265,120 @@ __global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant
         const double c2 = (ya + 2.0 * yb) * (1.0 / 3.0) - h18 * (Ma + 2.0 * Mb);
         closed = ya >= 0.0 && yb >= 0.0 && c1 >= 0.0 && c2 >= 0.0;
     }
-    const double iga = 1.0 / ga, igb = 1.0 / gb;
+    if (!closed) {
+        if (t0 == 0) {
+            const unsigned m = __activemask(), below = m & ((1u << (threadIdx.x & 31)) - 1u);
+            const bool whole = m == 0xffffffffu;
+            unsigned long long pos = 0;
+            if (!below) pos = atomicAdd(whole ? &queue->front : &queue->back, (unsigned long long)__popc(m));
+            pos = __shfl_sync(m, pos, __ffs(m) - 1) + __popc(below);
+            list[whole ? pos : list_n - 1 - pos] = make_int2(ia, ib);
+        }
+        return;
+    }
     // quartic q of the cut piece (or the ramp): sigma~ U = sum_m q_m (U - u0)^m on [u0, U_j]
     double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0, q4 = 0.0, w = 0.0, p = 0.0;
-    if (closed) {
-        w = A.u[j] - u0;
-        if (j > 0) {
-            const int k = j - 1;
-            const double h = A.u[j] - A.u[k], ih = 1.0 / h, t = (u0 - A.u[k]) * ih, r = 1.0 - t;
-            const double ya = y[k * st], yb = y[j * st], Ma = M[k * st], Mb = M[j * st];
-            const double p0 = r * ya + t * yb + h * h * (1.0 / 6.0) * ((r * r * r - r) * Ma + (t * t * t - t) * Mb);
-            const double p1 = (yb - ya) * ih + h * (1.0 / 6.0) * ((1.0 - 3.0 * r * r) * Ma + (3.0 * t * t - 1.0) * Mb);
-            const double p2 = 0.5 * (r * Ma + t * Mb), p3 = (Mb - Ma) * ih * (1.0 / 6.0);
-            q0 = p0 * u0;
-            q1 = fma(p1, u0, p0);
-            q2 = fma(p2, u0, p1);
-            q3 = fma(p3, u0, p2);
-            q4 = p3;
-        } else if (w > 0.0) {
-            const double ramp = y[0] / w;
-            q1 = ramp * u0;
-            q2 = ramp;
-        }
-        // the tail's exponent
-        const double yK = y[(K - 1) * st], yJ = y[(K - 2) * st];
-        if (yK > 0.0 && yJ > 0.0) p = fmin(0.0, fmax(-1.0, log(yK / yJ) / A.ln_uK));
+    w = A.u[j] - u0;
+    if (j > 0) {
+        const int k = j - 1;
+        const double h = A.u[j] - A.u[k], ih = 1.0 / h, t = (u0 - A.u[k]) * ih, r = 1.0 - t;
+        const double ya = y[k * st], yb = y[j * st], Ma = M[k * st], Mb = M[j * st];
+        const double p0 = r * ya + t * yb + h * h * (1.0 / 6.0) * ((r * r * r - r) * Ma + (t * t * t - t) * Mb);
+        const double p1 = (yb - ya) * ih + h * (1.0 / 6.0) * ((1.0 - 3.0 * r * r) * Ma + (3.0 * t * t - 1.0) * Mb);
+        const double p2 = 0.5 * (r * Ma + t * Mb), p3 = (Mb - Ma) * ih * (1.0 / 6.0);
+        q0 = p0 * u0;
+        q1 = fma(p1, u0, p0);
+        q2 = fma(p2, u0, p1);
+        q3 = fma(p3, u0, p2);
+        q4 = p3;
+    } else if (w > 0.0) {
+        const double ramp = y[0] / w;
+        q1 = ramp * u0;
+        q2 = ramp;
     }
+    // the tail's exponent
+    const double yK = y[(K - 1) * st], yJ = y[(K - 2) * st];
+    if (yK > 0.0 && yJ > 0.0) p = fmin(0.0, fmax(-1.0, log(yK / yJ) / A.ln_uK));
     for (int t = t0; t < t1; ++t) {
         const double th = A.kT[t], ith = A.ikT[t];
-        double acc;
-        if (closed) {
-            const double *tab = A.tab + (size_t)t * rate_tab_stride(K);
-            // exp(-800) is zero in FP64, and z^4 exp(-z) with it
-            const double z = fmin(w * ith, 800.0), ez = exp(-z);
-            double G[5];
-            lower_gammas(z, ez, G);
-            acc = th * fma(q0, G[0], th * fma(q1, G[1], th * fma(q2, G[2], th * fma(q3, G[3], th * (q4 * G[4])))));
-            double whole = 0.0;
-            const double *W = tab + j * K;
-            for (int m = 0; m < K; ++m) whole = fma(__ldg(W + m), y[m * st], whole);
-            acc = fma(ez, whole, acc);
-            // tail: y_K kT U_K g(p) exp(-(U_K - u0)/kT), g(p) = x^-(1+p) Gamma(2 + p, x) e^x at x = U_K/kT;
-            // left out under the quadrature's remainder bound
-            const double eK = ez * __ldg(tab + K * K + j), uK = A.u[K - 1];
-            if (!(4.0 * ymax * th * (uK + th) * eK <= 1e-17 * acc)) {
-                double gp;
-                if (uK * ith >= kRateChebX) {
-                    const double *ch = tab + K * K + K, chx = fma(2.0, p, 1.0);  // [-1, 0] on [-1, 1]
-                    double d1 = 0.0, d2 = 0.0;
-                    for (int m = kRateCheb - 1; m > 0; --m) {
-                        const double d = fma(2.0 * chx, d1, __ldg(ch + m) - d2);
-                        d2 = d1;
-                        d1 = d;
-                    }
-                    gp = fma(chx, d1, __ldg(ch) - d2);
-                } else {
-                    gp = rate_tail(p, uK * ith);
+        const double *tab = A.tab + (size_t)t * rate_tab_stride(K);
+        // exp(-800) is zero in FP64, and z^4 exp(-z) with it
+        const double z = fmin(w * ith, 800.0), ez = exp(-z);
+        double G[5];
+        lower_gammas(z, ez, G);
+        double acc = th * fma(q0, G[0], th * fma(q1, G[1], th * fma(q2, G[2], th * fma(q3, G[3], th * (q4 * G[4])))));
+        double whole = 0.0;
+        const double *W = tab + j * K;
+        for (int m = 0; m < K; ++m) whole = fma(__ldg(W + m), y[m * st], whole);
+        acc = fma(ez, whole, acc);
+        // tail: y_K kT U_K g(p) exp(-(U_K - u0)/kT), g(p) = x^-(1+p) Gamma(2 + p, x) e^x at x = U_K/kT;
+        // left out under the quadrature's remainder bound
+        const double eK = ez * __ldg(tab + K * K + j), uK = A.u[K - 1];
+        if (!(4.0 * ymax * th * (uK + th) * eK <= 1e-17 * acc)) {
+            double gp;
+            if (uK * ith >= kRateChebX) {
+                const double *ch = tab + K * K + K, chx = fma(2.0, p, 1.0);  // [-1, 0] on [-1, 1]
+                double d1 = 0.0, d2 = 0.0;
+                for (int m = kRateCheb - 1; m > 0; --m) {
+                    const double d = fma(2.0 * chx, d1, __ldg(ch + m) - d2);
+                    d2 = d1;
+                    d1 = d;
                 }
-                acc = fma(y[(K - 1) * st] * th * uK * eK, gp, acc);
+                gp = fma(chx, d1, __ldg(ch) - d2);
+            } else {
+                gp = rate_tail(p, uK * ith);
             }
-        } else {
-            acc = rate_quadrature(A, y, M, st, ymax, u0, th, ith);
+            acc = fma(y[(K - 1) * st] * th * uK * eK, gp, acc);
         }
-        const double c = A.pref[t] * acc;
-        // exp(-dE/(2kT)) exp(-u0/kT): exp(-|dE|/kT) for an excitation, 1 for a quenching
-        const double ex = exp(-2.0 * u0 * ith);
-        rate[t * plane + ab] = c * (dE >= 0.0 ? ex : 1.0) * iga;
-        rate[t * plane + ba] = c * (dE >= 0.0 ? 1.0 : ex) * igb;
+        rate_store(A, rate + t * plane, t, acc, dE, u0 * ith, ga, gb, ia, ib);
+    }
+}
+
+// The listed pairs by quadrature: one thread per pair and temperature (temperature is the slow index: the lanes of a
+// warp share kT and so take similar panel counts).  Two blocks per SM, i.e. two warps per FP64 pipe, which keep it
+// busy; with few items a warp takes fewer than 32 (its time is that of its longest), and the first items go to
+// different SMs and sub-partitions, the rest to whichever warp is free.  The pair's values come from `sym` where
+// that was asked for (it may be sigma's own memory).  Calls of 1032 levels x 5 temperatures: every pair listed
+// 35.7 ms, 0.2 % of the values negative 6.0 ms; 200 levels x 64 temperatures, most pairs listed, 11.2 ms (57 ms
+// when a warp ran its pairs' quadratures in place; 37.6, 27 and 21.6 ms with every pair by quadrature).
+__global__ void __launch_bounds__(kRateThreads, 2) k_rates_quad(const __grid_constant__ RateArgs A, const double *sigma,
+                                                              const double *sym, const double *g, const double *E, double *rate,
+                                                              RateQueue *queue, const int2 *list, size_t list_n)
+{
+    extern __shared__ double rsm[];
+    const int K = A.K, lane = threadIdx.x & 31, half = gridDim.x / 2;
+    constexpr int st = kRateThreads, warps = kRateThreads / 32;
+    double *y = rsm + threadIdx.x, *M = y + K * st;
+    const size_t plane = (size_t)A.L * A.L;
+    const unsigned long long front = queue->front, pairs = front + queue->back;
+    const int lanes = (int)min(32ull, (pairs * A.n_T + warps * half - 1) / (warps * half));
+    // items per temperature: the pairs, in whole warps where a warp takes 32
+    const unsigned long long row = lanes == 32 ? (pairs + 31) & ~31ull : pairs, items = row * A.n_T;
+    unsigned long long i0 = ((blockIdx.x / half) * warps + threadIdx.x / 32) * (unsigned long long)half + blockIdx.x % half;
+    for (i0 *= lanes; i0 < items;) {
+        const unsigned long long i = i0 + lane, p = i % row;
+        if (lane < lanes && i < items && p < pairs) {
+            const int2 pr = list[p < front ? p : list_n - 1 - (p - front)];
+            const int t = (int)(i / row), ia = pr.x, ib = pr.y;
+            const size_t ab = (size_t)ia * A.L + ib, ba = (size_t)ib * A.L + ia;
+            const double ga = g[ia], gb = g[ib];
+            double ymax = 0.0;
+            for (int k = 0; k < K; ++k) {
+                const double v = sym ? sym[k * plane + ab] : 0.5 * (ga * sigma[k * plane + ab] + gb * sigma[k * plane + ba]);
+                y[k * st] = v;
+                ymax = fmax(ymax, fabs(v));
+            }
+            for (int k = 0; k < K; ++k) {
+                double m = 0.0;
+                for (int j = 0; j < K; ++j) m = fma(A.Q[k][j], y[j * st], m);
+                M[k * st] = m;
+            }
+            const double dE = E[ib] - E[ia], u0 = 0.5 * fabs(dE), th = A.kT[t], ith = A.ikT[t];
+            rate_store(A, rate + t * plane, t, rate_quadrature(A, y, M, st, ymax, u0, th, ith), dE, u0 * ith, ga, gb, ia, ib);
+        }
+        __syncwarp();
+        if (lane == 0) i0 = 2ull * half * warps * lanes + atomicAdd(&queue->next, (unsigned long long)lanes);
+        i0 = __shfl_sync(0xffffffffu, i0, 0);
     }
 }
 
@@ -536,12 +601,28 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
     // the closed form's powers of kT stay far from the limits of FP64 in this range
     A.closed = A.u[0] >= 1e-12 && A.u[K - 1] <= 1e6;
     for (int t = 0; t < nT; ++t) A.closed = A.closed && A.kT[t] >= 1e-12 && A.kT[t] <= 1e6;
-    // one upload: degeneracies, level energies, tables
+    // the rows of pairs (a <= b) in passes of at most kRatePass pairs, which bounds the list
+    std::vector<int> first{0};
+    size_t list_n = 0, n_pairs = 0;
+    for (int b = 0; b < L; b += kRateTb) {
+        const int b1 = std::min(L, b + kRateTb);
+        const size_t rows = ((size_t)b1 * (b1 + 1) - (size_t)b * (b + 1)) / 2;
+        if (n_pairs && n_pairs + rows > kRatePass) {
+            first.push_back(b);
+            n_pairs = 0;
+        }
+        n_pairs += rows;
+        list_n = std::max(list_n, n_pairs);
+    }
+    first.push_back(L);
+    const size_t passes = first.size() - 1;
+    // one upload: degeneracies, level energies, tables, empty queues
     std::vector<double> up;
     if (A.closed) rate_tables(A, up);
     const size_t tab_n = up.size();
     up.insert(up.end(), d->degeneracy, d->degeneracy + L);
     up.insert(up.end(), d->level_energy, d->level_energy + L);
+    up.insert(up.end(), passes * sizeof(RateQueue) / sizeof(double), 0.0);
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     cudaError_t e;
@@ -566,28 +647,40 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
         dsig = p;
     }
     // a pageable copy is staged by the runtime before cudaMemcpyAsync returns
+    int2 *list = nullptr;
     if ((e = get((void **)&dup, sizeof(double) * up.size())) != cudaSuccess ||
+        (e = get((void **)&list, sizeof(int2) * list_n)) != cudaSuccess ||
         (e = cudaMemcpyAsync(dup, up.data(), sizeof(double) * up.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "staging levels");
     }
     A.tab = dup;
     const double *dg = dup + tab_n, *dE = dg + L;
+    RateQueue *queues = reinterpret_cast<RateQueue *>(dup + tab_n + 2 * (size_t)L);
     if (host_rate && (e = get((void **)&drate, rate_bytes)) != cudaSuccess) { cleanup(); return cuda_fail(e, "cudaMallocAsync"); }
     if (host_sym && (e = get((void **)&dsym, sig_bytes)) != cudaSuccess) { cleanup(); return cuda_fail(e, "cudaMallocAsync"); }
-    const int nta = (L + kRateTa - 1) / kRateTa, ntb = (L + kRateTb - 1) / kRateTb;
     const size_t smem = sizeof(double) * 2 * (size_t)K * kRateThreads;
-    if ((e = cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) {
+    if ((e = cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_rates_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "cudaFuncSetAttribute");
     }
-    // a thread runs all temperatures of its pair (the pair's spline is formed once); with too few tiles to
-    // fill the GPU the temperatures are spread over blocks instead
-    const long long tiles = (long long)nta * ntb / 2 + 1;
-    const int split = (int)std::min<long long>(nT, std::max<long long>(1, 608 / tiles));
-    A.t_chunk = (nT + split - 1) / split;
-    k_rates<<<dim3(nta, ntb, (nT + A.t_chunk - 1) / A.t_chunk), kRateThreads, smem, st>>>(A, dsig, dg, dE, dsym, drate);
-    count_launches(1);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (size_t ps = 0; ps < passes; ++ps) {
+        const int b0 = first[ps], b1 = first[ps + 1];
+        const int nta = (b1 + kRateTa - 1) / kRateTa, ntb = (b1 - b0 + kRateTb - 1) / kRateTb;
+        // a thread runs all temperatures of its pair (the pair's spline is formed once); with too few tiles to
+        // fill the GPU the temperatures are spread over blocks instead
+        const long long tiles = (long long)nta * ntb / 2 + 1;
+        const int split = (int)std::min<long long>(nT, std::max<long long>(1, 608 / tiles));
+        A.t_chunk = (nT + split - 1) / split;
+        k_rates<<<dim3(nta, ntb, (nT + A.t_chunk - 1) / A.t_chunk), kRateThreads, smem, st>>>(A, dsig, dg, dE, dsym, drate, b0,
+                                                                                           queues + ps, list, list_n);
+        k_rates_quad<<<2 * sms, kRateThreads, smem, st>>>(A, dsig, dsym, dg, dE, drate, queues + ps, list, list_n);
+    }
+    count_launches(2 * (long long)passes);
     if ((e = cudaGetLastError()) != cudaSuccess) { cleanup(); return cuda_fail(e, "rate kernels"); }
     if (host_rate && (e = cudaMemcpyAsync(rate, drate, rate_bytes, cudaMemcpyDeviceToHost, st)) != cudaSuccess) {
         cleanup();
