@@ -489,8 +489,9 @@ void host_gammas(double z, double G[5])
         }
         return;
     }
+    // as many terms as z needs (the first one left out is below 1e-21)
     double s = 1.0;
-    for (int n = 60; n >= 6; --n) s = 1.0 + s * z / n;
+    for (int n = std::min(60, 18 + (int)(6.0 * z)); n >= 6; --n) s = 1.0 + s * z / n;
     double zm = z * z * z * z;
     G[4] = 0.2 * s * zm * z * ez;
     for (int m = 4; m >= 1; --m) {
@@ -505,6 +506,11 @@ void rate_tables(const RateArgs &A, std::vector<double> &tab)
     const int K = A.K, stride = rate_tab_stride(K);
     tab.assign((size_t)A.n_T * stride, 0.0);
     const double pi = 3.14159265358979323846;
+    double node[kRateCheb], cosine[kRateCheb][kRateCheb];  // the Chebyshev points and the series' cosines there
+    for (int i = 0; i < kRateCheb; ++i) {
+        node[i] = std::cos(pi * (i + 0.5) / kRateCheb);
+        for (int m = 0; m < kRateCheb; ++m) cosine[m][i] = std::cos(pi * m * (i + 0.5) / kRateCheb);
+    }
     for (int t = 0; t < A.n_T; ++t) {
         double *W = tab.data() + (size_t)t * stride, *eK = W + K * K, *ch = eK + K;
         const double th = A.kT[t], uK = A.u[K - 1];
@@ -533,10 +539,10 @@ void rate_tables(const RateArgs &A, std::vector<double> &tab)
         if (uK / th < 0.5 * kRateChebX) continue;  // not read (half: whatever the rounding of the kernel's ratio)
         double f[kRateCheb];
         for (int i = 0; i < kRateCheb; ++i)
-            f[i] = upper_gamma_reduced(1.5 + 0.5 * std::cos(pi * (i + 0.5) / kRateCheb), uK / th);
+            f[i] = upper_gamma_reduced(1.5 + 0.5 * node[i], uK / th);
         for (int m = 0; m < kRateCheb; ++m) {
             double c = 0.0;
-            for (int i = 0; i < kRateCheb; ++i) c += f[i] * std::cos(pi * m * (i + 0.5) / kRateCheb);
+            for (int i = 0; i < kRateCheb; ++i) c += f[i] * cosine[m][i];
             ch[m] = c * (m ? 2.0 : 1.0) / kRateCheb;
         }
     }

@@ -77,3 +77,25 @@ def test_listed_pairs_do_not_hold_the_others():
             times.append(time.perf_counter() - t0)
         best.append(min(times))
     assert best[1] < 1.2 * best[0]
+
+
+def test_temperatures_cost_little_on_the_host():
+    """A temperature adds its tables on the host and its kernel time to a call with five levels, far less than the
+    microseconds that a temperature takes when every cosine of its series is evaluated anew."""
+    import torch
+
+    import paper_2312_02322_gb300.api as mq
+
+    def best(nt):
+        rs = W.rate_set(n_levels=5, temps_k=tuple(np.geomspace(10, 2000, nt)))
+        dev = torch.from_numpy(rs.sigma).cuda()
+        times = []
+        for _ in range(30):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            mq.rate_coefficients(dev, rs.u, rs.energy, rs.g, rs.mu, rs.kT)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t0)
+        return min(times)
+
+    assert (best(256) - best(1)) / 255 < 3e-6
