@@ -466,12 +466,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_stage(TcState T, int s, in
 //   w = sum_c M_rc(x) C_c,   u = (dx/dR) sum_c M'_rc(x) C_c,
 // then the element update of Eq. 5 and RK4 (every load coalesced over the slots) and the per-slot
 // partial sums of force, torque and diagnostics over the 256 rows (compensated FP32 across warps).
-// Bound by the latency of its gathers: five CTAs per SM (48 registers, 28 spilled loads outside the loop over
+// Bound by the latency of its gathers: five CTAs per SM (MINB; 48 registers, spilled loads outside the loop over
 // the non-zeros) hide more of it than four with 64: N = 40401, 512 slots 142.8 -> 138.1 ms for 48 steps, 1024 slots
-// 244.6 -> 237.0 ms; six gain nothing more (133 and 245 ms).
+// 244.6 -> 237.0 ms; six gain nothing more (133 and 245 ms).  A grid that four CTAs per SM hold takes the form without
+// spills: N = 1681, 100 slots 6.44 -> 5.65 ms for 16 steps, 2048 slots (448 CTAs) 11.03 -> 9.53 ms; N = 10201, 256
+// slots (320 CTAs) 10.39 -> 8.81 ms.
 constexpr int kSpWarps = 8, kSpTile = 32;
 
-__global__ void __launch_bounds__(32 * kSpWarps, 5) k_sp_stage(TcState T, int s, int cur)
+template <int MINB>
+__global__ void __launch_bounds__(32 * kSpWarps, MINB) k_sp_stage(TcState T, int s, int cur)
 {
     const DevSys &S = *T.sys;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1148,7 +1151,9 @@ mqct_status run_tc_batched(const BatchArgs &a, const DevSys &h, cudaStream_t st)
     };
     // the stage kernel: tcgen05 contraction (factorised BF16X3) or the sparse FP32 table (PLAIN)
     auto stage = [&](cudaStream_t q, int s, int cur) {
-        if (plain) k_sp_stage<<<dim3(S / kSpTile, n_rowblocks), 32 * kSpWarps, 0, q>>>(T, s, cur);
+        const dim3 sp(S / kSpTile, n_rowblocks);
+        if (plain && (long long)sp.x * sp.y <= 4ll * sms) k_sp_stage<4><<<sp, 32 * kSpWarps, 0, q>>>(T, s, cur);
+        else if (plain) k_sp_stage<5><<<sp, 32 * kSpWarps, 0, q>>>(T, s, cur);
         else k_tc_stage<<<h.n_tiles * n_ct, kTcThreads, smem, q>>>(T, s, cur);
     };
     // PLAIN path: the slots sorted by interval at the end of each chunk
