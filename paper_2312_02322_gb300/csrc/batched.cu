@@ -978,6 +978,7 @@ int batched_slots(const DevSys &h, size_t cap)
 {
     constexpr int NE = T / 32 - batch_slot_warps(BMAX);
     constexpr size_t kMaxBytes = 232448;  // shared memory of a CTA
+    static_assert(kUpt * NE * 32 <= kBatchMaxRows, "the group tables are built for at most kBatchMaxRows rows");
     const size_t n = h.n, nl = h.n_levels, L = h.L;
     for (int b = BMAX; b >= 4; b >>= 1) {
         const size_t bound = 24 * (n + nl) * b + 16 * L * b + 4 * nl + 32 * (size_t)NE * b + 16 + 400 + 200 * BMAX;

@@ -21,6 +21,7 @@ inline __host__ __device__ dbl4 make_dbl4(double x, double y, double z, double w
 constexpr int kSlice = 32;     // rows per SELL slice (one warp)
 constexpr int kMaxTerms = 64;  // expansion terms held in shared memory per stage
 constexpr int kMaxWarps = 32;
+constexpr int kBatchMaxRows = 1920;  // rows of the largest basis that a shape of the FP32 batched kernel takes
 
 // Device view of one system; an array of these lives in device memory so that one
 // persistent launch can serve trajectories of several systems (uneven basis sizes).

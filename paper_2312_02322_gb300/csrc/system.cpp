@@ -573,37 +573,39 @@ extern "C" mqct_status mqct_create_system(const mqct_system_desc *d, mqct_system
                 vf[i] = make_float4((float)vcoef[i].x, (float)vcoef[i].y, (float)vcoef[i].z, (float)vcoef[i].w);
             std::vector<float> aupf(aup.begin(), aup.end()), adnf(adn.begin(), adn.end());
             up_(fvalf, &D.f_valf);
-            if (d->precision == MQCT_FP32 && n <= 0xffff) {
+            if (d->precision == MQCT_FP32 && n <= kBatchMaxRows) {
                 // groups of two terms whose non-zeros share columns: pairs in the order of the
                 // entries they save, a pair only when its union has at most 3/4 of the entries of the two
                 const int nf = (int)fterm.size();
-                auto merged = [&](int fa, int fb, int r) {
-                    std::vector<int> c;
-                    for (auto &e2 : grows[fterm[fa]][r]) c.push_back(e2.c);
-                    if (fb >= 0)
-                        for (auto &e2 : grows[fterm[fb]][r]) c.push_back(e2.c);
-                    std::sort(c.begin(), c.end());
-                    c.erase(std::unique(c.begin(), c.end()), c.end());
-                    return c;
-                };
+                std::vector<long long> count(nf, 0), shared((size_t)nf * nf, 0);
+                {
+                    // per row, the terms of every column (L <= 64)
+                    std::vector<unsigned long long> mask(n, 0);
+                    std::vector<int> touched;
+                    for (int r = 0; r < n; ++r) {
+                        touched.clear();
+                        for (int f = 0; f < nf; ++f) {
+                            count[f] += (long long)grows[fterm[f]][r].size();
+                            for (auto &e : grows[fterm[f]][r]) {
+                                if (!mask[e.c]) touched.push_back(e.c);
+                                mask[e.c] |= 1ull << f;
+                            }
+                        }
+                        for (int c : touched) {
+                            for (unsigned long long m = mask[c]; m; m &= m - 1) {
+                                const int fa = __builtin_ctzll(m);
+                                for (unsigned long long m2 = m & (m - 1); m2; m2 &= m2 - 1) ++shared[(size_t)fa * nf + __builtin_ctzll(m2)];
+                            }
+                            mask[c] = 0;
+                        }
+                    }
+                }
                 struct Pair { long long save; int a, b; };
                 std::vector<Pair> cand;
                 for (int fa = 0; fa < nf; ++fa)
                     for (int fb = fa + 1; fb < nf; ++fb) {
-                        long long sum = 0, uni = 0;
-                        for (int r = 0; r < n; ++r) {
-                            // entries of a row are in ascending column order
-                            const auto &ea = grows[fterm[fa]][r], &eb = grows[fterm[fb]][r];
-                            size_t ia = 0, ib = 0, shared = 0;
-                            while (ia < ea.size() && ib < eb.size()) {
-                                if (ea[ia].c == eb[ib].c) { ++shared; ++ia; ++ib; }
-                                else if (ea[ia].c < eb[ib].c) ++ia;
-                                else ++ib;
-                            }
-                            sum += (long long)(ea.size() + eb.size());
-                            uni += (long long)(ea.size() + eb.size() - shared);
-                        }
-                        if (4 * uni <= 3 * sum) cand.push_back({sum - uni, fa, fb});
+                        const long long sum = count[fa] + count[fb], save = shared[(size_t)fa * nf + fb];
+                        if (4 * (sum - save) <= 3 * sum) cand.push_back({save, fa, fb});
                     }
                 std::stable_sort(cand.begin(), cand.end(), [](const Pair &x, const Pair &y) { return x.save > y.save; });
                 std::vector<int> mate(nf, -1);
@@ -612,41 +614,46 @@ extern "C" mqct_status mqct_create_system(const mqct_system_desc *d, mqct_system
                 std::vector<std::pair<int, int>> grp;
                 for (int f = 0; f < nf; ++f)
                     if (mate[f] < 0 || mate[f] > f) grp.push_back({f, mate[f]});
-                D.n_grp = (int)grp.size();
-                std::vector<int> grow(L, -1), goff(n_slices), gwidth((size_t)n_slices * std::max<size_t>(1, grp.size()), 0);
+                const size_t ng = grp.size();
+                D.n_grp = (int)ng;
+                std::vector<int> grow(L, -1), goff(n_slices), gwidth((size_t)n_slices * std::max<size_t>(1, ng), 0);
                 std::vector<float2> gval;
                 std::vector<uint16_t> gcol;
-                auto value = [&](int f, int r, int c) -> float {
-                    if (f >= 0)
-                        for (auto &e2 : grows[fterm[f]][r])
-                            if (e2.c == c) return (float)e2.v;
-                    return 0.f;
-                };
-                auto put = [&](int c, float va, float vb) {
-                    gcol.push_back((uint16_t)c);
-                    gval.push_back(make_float2(va, vb));
-                };
-                for (size_t g = 0; g < grp.size(); ++g) {
+                for (size_t g = 0; g < ng; ++g) {
                     grow[fterm[grp[g].first]] = 2 * (int)g;
                     if (grp[g].second >= 0) grow[fterm[grp[g].second]] = 2 * (int)g + 1;
                 }
+                struct Merged { int c; float a, b; };
+                std::vector<Merged> row[kSlice];
+                const std::vector<Entry> none;
                 for (int sl = 0; sl < n_slices; ++sl) {
                     goff[sl] = (int)gval.size();
-                    for (size_t g = 0; g < grp.size(); ++g) {
-                        std::vector<std::vector<int>> cols(kSlice);
+                    for (size_t g = 0; g < ng; ++g) {
                         size_t width = 0;
-                        for (int q = 0; q < kSlice && sl * kSlice + q < n; ++q) {
-                            cols[q] = merged(grp[g].first, grp[g].second, sl * kSlice + q);
-                            width = std::max(width, cols[q].size());
+                        for (int q = 0; q < kSlice; ++q) {
+                            // the union of the two terms' columns (a row's entries are in ascending column order)
+                            row[q].clear();
+                            const int r = sl * kSlice + q;
+                            if (r >= n) continue;
+                            const auto &ea = grows[fterm[grp[g].first]][r], &eb = grp[g].second >= 0 ? grows[fterm[grp[g].second]][r] : none;
+                            size_t ia = 0, ib = 0;
+                            while (ia < ea.size() || ib < eb.size()) {
+                                const int ca = ia < ea.size() ? ea[ia].c : n, cb = ib < eb.size() ? eb[ib].c : n, c = std::min(ca, cb);
+                                row[q].push_back({c, ca == c ? (float)ea[ia].v : 0.f, cb == c ? (float)eb[ib].v : 0.f});
+                                ia += ca == c;
+                                ib += cb == c;
+                            }
+                            width = std::max(width, row[q].size());
                         }
-                        gwidth[(size_t)sl * grp.size() + g] = (int)width | (grp[g].second >= 0 ? 1 << 16 : 0);
+                        gwidth[(size_t)sl * ng + g] = (int)width | (grp[g].second >= 0 ? 1 << 16 : 0);
+                        size_t o = gval.size();
+                        gval.resize(o + width * kSlice);
+                        gcol.resize(o + width * kSlice);
                         for (size_t k = 0; k < width; ++k)
-                            for (int q = 0; q < kSlice; ++q) {
-                                const int r = std::min(sl * kSlice + q, n - 1);
-                                if (k < cols[q].size())
-                                    put(cols[q][k], value(grp[g].first, r, cols[q][k]), value(grp[g].second, r, cols[q][k]));
-                                else
-                                    put(r, 0.f, 0.f);  // padding: the row itself, zero values
+                            for (int q = 0; q < kSlice; ++q, ++o) {
+                                const bool in = k < row[q].size();  // else padding: the row itself, zero values
+                                gcol[o] = (uint16_t)(in ? row[q][k].c : std::min(sl * kSlice + q, n - 1));
+                                gval[o] = in ? make_float2(row[q][k].a, row[q][k].b) : make_float2(0.f, 0.f);
                             }
                     }
                 }
@@ -657,12 +664,26 @@ extern "C" mqct_status mqct_create_system(const mqct_system_desc *d, mqct_system
                     std::memcpy(&db, &adnf[r], sizeof db);
                     rinfo[r] = make_int4((int)((unsigned)up[r] | ((unsigned)dn[r] << 16)), S.lev[r], ub, db);
                 }
-                up_(grow, &D.grp_row);
-                up_(goff, &D.g_off);
-                up_(gwidth, &D.g_width);
-                up_(gval, &D.g_val);
-                up_(gcol, &D.g_col);
-                up_(rinfo, &D.row_info);
+                // one device buffer for all of them
+                std::vector<int4> buf;
+                auto place = [&](const auto &v) {
+                    const size_t o = buf.size(), bytes = sizeof(v[0]) * v.size();
+                    buf.resize(o + (bytes + sizeof(int4) - 1) / sizeof(int4), make_int4(0, 0, 0, 0));
+                    if (bytes) std::memcpy(buf.data() + o, v.data(), bytes);
+                    return o;
+                };
+                const size_t o_info = place(rinfo), o_val = place(gval), o_off = place(goff), o_width = place(gwidth),
+                             o_row = place(grow), o_col = place(gcol);
+                const int4 *base = nullptr;
+                up_(buf, &base);
+                if (st == MQCT_OK) {
+                    D.row_info = base + o_info;
+                    D.g_val = reinterpret_cast<const float2 *>(base + o_val);
+                    D.g_off = reinterpret_cast<const int *>(base + o_off);
+                    D.g_width = reinterpret_cast<const int *>(base + o_width);
+                    D.grp_row = reinterpret_cast<const int *>(base + o_row);
+                    D.g_col = reinterpret_cast<const unsigned short *>(base + o_col);
+                }
             }
             up_(aupf, &D.aupf);
             up_(adnf, &D.adnf);
