@@ -68,15 +68,6 @@ enum { SLOT_IDLE = 0, SLOT_ACTIVE = 1, SLOT_FINAL = 2, SLOT_WAIT = 3 };
 __host__ __device__ constexpr int batch_slot_warps(int B) { return B > 8 ? B / 8 : 1; }
 
 // ---- packed arithmetic on two slots (each half rounded as the scalar instruction)
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
-          "l"(reinterpret_cast<const unsigned long long &>(c)));
-    return d;
-}
 __device__ __forceinline__ float2 mul2(float2 a, float2 b)
 {
     float2 d;

@@ -40,17 +40,6 @@ constexpr long long kTcWait = 1ll << 24;
 
 enum { TS_IDLE = 0, TS_ACTIVE = 1, TS_FINAL = 2, TS_WAIT = 3 };
 
-// packed FP32 fused multiply-add, each half rounded as the scalar instruction
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
-          "l"(reinterpret_cast<const unsigned long long &>(c)));
-    return d;
-}
-
 // per-slot values that are not per component (the four component lanes of a slot read them)
 struct TSlot {
     double dt, h6, r_end, e0, j0, ndev, edev, jdev;

@@ -81,6 +81,17 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// fused multiply-add on packed pairs, each half rounded as the scalar instruction
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+          "l"(reinterpret_cast<const unsigned long long &>(c)));
+    return d;
+}
+
 // comparisons that keep off the FP64 pipe: for a finite x >= 0 and y >= 0, x >= y compares the bit
 // patterns; a double is finite unless its exponent bits are all ones
 __device__ __forceinline__ bool ge_pos(double x, double y)
