@@ -79,6 +79,9 @@ struct RateQueue {
     unsigned long long front, back, next, pad;
 };
 
+// tiles before row j of tiles (eight levels b): row i has those a-tiles (16 levels) with a <= 8 i + 7, i / 2 + 1 of them
+__host__ __device__ constexpr long long rate_tiles(long long j) { return (j / 2) * (j / 2 + 1) + (j % 2) * (j / 2 + 1); }
+
 // doubles of A.tab per temperature
 __host__ __device__ constexpr int rate_tab_stride(int K) { return K * K + K + kRateCheb; }
 
@@ -222,24 +225,29 @@ __device__ __forceinline__ void rate_store(const RateArgs &A, double *rate, int 
 
 // One thread per unordered pair (a <= b): the symmetrised cross sections of Eq. 20 (sym, or NULL) and, where the
 // closed form holds, both rates; the other pairs join the list that k_rates_quad integrates, so that no thread waits
-// for a quadrature.  A block takes a tile of 16 x 8 pairs (rows from b_first on), so that the transposed reads
-// sigma[k][a][b] of its warps share 32-byte sectors.  Bound by the FP64 pipe: a call with 1032 levels x 10 energies x
-// 5 temperatures, all in closed form, takes 1.26 ms (the kernel 0.94); with the quadrature of every pair 27 ms.
+// for a quadrature.  A block takes a tile of 16 x 8 pairs, so that the transposed reads sigma[k][a][b] of its warps
+// share 32-byte sectors; only tiles with pairs a <= b have a block (rate_tiles), since the empty blocks of a
+// rectangular grid leave the others unevenly spread over the SMs.  Bound by the FP64 pipe: a call with 1032 levels x
+// 10 energies x 5 temperatures, all in closed form, takes 1.20 ms (the kernel 0.94); with the quadrature of every
+// pair 27 ms.
 __global__ void __launch_bounds__(kRateThreads, 3) k_rates(const __grid_constant__ RateArgs A, const double *sigma,
                                                          const double *g, const double *E, double *sym, double *rate,
-                                                         int b_first, RateQueue *queue, int2 *list, size_t list_n)
+                                                         long long first, RateQueue *queue, int2 *list, size_t list_n)
 {
     extern __shared__ double rsm[];
     const int K = A.K, L = A.L;
-    const int a0 = blockIdx.x * kRateTa, b0 = b_first + blockIdx.y * kRateTb;
-    if (a0 > b0 + kRateTb - 1) return;
-    const int ia = a0 + threadIdx.x % kRateTa, ib = b0 + threadIdx.x / kRateTa;
+    // tile first + blockIdx.x: row j of tiles is the last one with rate_tiles(j) at or below it
+    const long long tile = first + blockIdx.x;
+    long long j8 = (long long)sqrtf(4.f * (float)tile);
+    while (rate_tiles(j8) > tile) --j8;
+    while (rate_tiles(j8 + 1) <= tile) ++j8;
+    const int ia = (int)(tile - rate_tiles(j8)) * kRateTa + threadIdx.x % kRateTa, ib = (int)j8 * kRateTb + threadIdx.x / kRateTa;
     if (ia >= L || ib >= L || ia > ib) return;
     constexpr int st = kRateThreads;
     double *y = rsm + threadIdx.x, *M = y + K * st;
     const double ga = g[ia], gb = g[ib];
     const size_t plane = (size_t)L * L, ab = (size_t)ia * L + ib, ba = (size_t)ib * L + ia;
-    const int t0 = blockIdx.z * A.t_chunk, t1 = min(A.n_T, t0 + A.t_chunk);
+    const int t0 = blockIdx.y * A.t_chunk, t1 = min(A.n_T, t0 + A.t_chunk);
     double ymax = 0.0;
     for (int k = 0; k < K; ++k) {
         const double v = 0.5 * (ga * sigma[k * plane + ab] + gb * sigma[k * plane + ba]);
@@ -505,12 +513,19 @@ void rate_tables(const RateArgs &A, std::vector<double> &tab)
 {
     const int K = A.K, stride = rate_tab_stride(K);
     tab.assign((size_t)A.n_T * stride, 0.0);
-    const double pi = 3.14159265358979323846;
-    double node[kRateCheb], cosine[kRateCheb][kRateCheb];  // the Chebyshev points and the series' cosines there
-    for (int i = 0; i < kRateCheb; ++i) {
-        node[i] = std::cos(pi * (i + 0.5) / kRateCheb);
-        for (int m = 0; m < kRateCheb; ++m) cosine[m][i] = std::cos(pi * m * (i + 0.5) / kRateCheb);
-    }
+    // the Chebyshev points and the series' cosines there
+    struct Cheb {
+        double node[kRateCheb], cosine[kRateCheb][kRateCheb];
+        Cheb()
+        {
+            const double pi = 3.14159265358979323846;
+            for (int i = 0; i < kRateCheb; ++i) {
+                node[i] = std::cos(pi * (i + 0.5) / kRateCheb);
+                for (int m = 0; m < kRateCheb; ++m) cosine[m][i] = std::cos(pi * m * (i + 0.5) / kRateCheb);
+            }
+        }
+    };
+    static const Cheb cheb;
     for (int t = 0; t < A.n_T; ++t) {
         double *W = tab.data() + (size_t)t * stride, *eK = W + K * K, *ch = eK + K;
         const double th = A.kT[t], uK = A.u[K - 1];
@@ -539,10 +554,10 @@ void rate_tables(const RateArgs &A, std::vector<double> &tab)
         if (uK / th < 0.5 * kRateChebX) continue;  // not read (half: whatever the rounding of the kernel's ratio)
         double f[kRateCheb];
         for (int i = 0; i < kRateCheb; ++i)
-            f[i] = upper_gamma_reduced(1.5 + 0.5 * node[i], uK / th);
+            f[i] = upper_gamma_reduced(1.5 + 0.5 * cheb.node[i], uK / th);
         for (int m = 0; m < kRateCheb; ++m) {
             double c = 0.0;
-            for (int i = 0; i < kRateCheb; ++i) c += f[i] * cosine[m][i];
+            for (int i = 0; i < kRateCheb; ++i) c += f[i] * cheb.cosine[m][i];
             ch[m] = c * (m ? 2.0 : 1.0) / kRateCheb;
         }
     }
@@ -595,7 +610,13 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
             return fail(MQCT_ERR_INVALID_ARG, "mqct_rate_coefficients: degeneracies must be > 0, energies finite");
     }
     natural_spline_map(A.u, K, A.Q);
-    gauss_legendre(kGl, A.gx, A.gw);
+    struct Gauss {
+        double x[kGl], w[kGl];
+        Gauss() { gauss_legendre(kGl, x, w); }
+    };
+    static const Gauss gauss;
+    std::copy(gauss.x, gauss.x + kGl, A.gx);
+    std::copy(gauss.w, gauss.w + kGl, A.gw);
     for (int t = 0; t < nT; ++t) {
         A.ikT[t] = 1.0 / A.kT[t];
         A.pref[t] = std::sqrt(8.0 / (3.14159265358979323846 * d->mu)) * std::pow(A.kT[t], -1.5);
@@ -653,9 +674,7 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
         dsig = p;
     }
     // a pageable copy is staged by the runtime before cudaMemcpyAsync returns
-    int2 *list = nullptr;
-    if ((e = get((void **)&dup, sizeof(double) * up.size())) != cudaSuccess ||
-        (e = get((void **)&list, sizeof(int2) * list_n)) != cudaSuccess ||
+    if ((e = get((void **)&dup, sizeof(double) * up.size() + sizeof(int2) * list_n)) != cudaSuccess ||
         (e = cudaMemcpyAsync(dup, up.data(), sizeof(double) * up.size(), cudaMemcpyHostToDevice, st)) != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "staging levels");
@@ -663,11 +682,13 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
     A.tab = dup;
     const double *dg = dup + tab_n, *dE = dg + L;
     RateQueue *queues = reinterpret_cast<RateQueue *>(dup + tab_n + 2 * (size_t)L);
+    int2 *list = reinterpret_cast<int2 *>(dup + up.size());
     if (host_rate && (e = get((void **)&drate, rate_bytes)) != cudaSuccess) { cleanup(); return cuda_fail(e, "cudaMallocAsync"); }
     if (host_sym && (e = get((void **)&dsym, sig_bytes)) != cudaSuccess) { cleanup(); return cuda_fail(e, "cudaMallocAsync"); }
     const size_t smem = sizeof(double) * 2 * (size_t)K * kRateThreads;
-    if ((e = cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_rates_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) {
+    if (smem > 48 * 1024 &&  // what a launch may have without asking
+        ((e = cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+         (e = cudaFuncSetAttribute(k_rates_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)) {
         cleanup();
         return cuda_fail(e, "cudaFuncSetAttribute");
     }
@@ -675,15 +696,13 @@ extern "C" mqct_status mqct_rate_coefficients(const mqct_rate_desc *d, const dou
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (size_t ps = 0; ps < passes; ++ps) {
-        const int b0 = first[ps], b1 = first[ps + 1];
-        const int nta = (b1 + kRateTa - 1) / kRateTa, ntb = (b1 - b0 + kRateTb - 1) / kRateTb;
+        const long long tile0 = rate_tiles(first[ps] / kRateTb), tiles = rate_tiles((first[ps + 1] + kRateTb - 1) / kRateTb) - tile0;
         // a thread runs all temperatures of its pair (the pair's spline is formed once); with too few tiles to
         // fill the GPU the temperatures are spread over blocks instead
-        const long long tiles = (long long)nta * ntb / 2 + 1;
         const int split = (int)std::min<long long>(nT, std::max<long long>(1, 608 / tiles));
         A.t_chunk = (nT + split - 1) / split;
-        k_rates<<<dim3(nta, ntb, (nT + A.t_chunk - 1) / A.t_chunk), kRateThreads, smem, st>>>(A, dsig, dg, dE, dsym, drate, b0,
-                                                                                           queues + ps, list, list_n);
+        k_rates<<<dim3((unsigned)tiles, (nT + A.t_chunk - 1) / A.t_chunk), kRateThreads, smem, st>>>(A, dsig, dg, dE, dsym, drate,
+                                                                                                  tile0, queues + ps, list, list_n);
         k_rates_quad<<<2 * sms, kRateThreads, smem, st>>>(A, dsig, dsym, dg, dE, drate, queues + ps, list, list_n);
     }
     count_launches(2 * (long long)passes);
