@@ -664,26 +664,12 @@ extern "C" mqct_status mqct_create_system(const mqct_system_desc *d, mqct_system
                     std::memcpy(&db, &adnf[r], sizeof db);
                     rinfo[r] = make_int4((int)((unsigned)up[r] | ((unsigned)dn[r] << 16)), S.lev[r], ub, db);
                 }
-                // one device buffer for all of them
-                std::vector<int4> buf;
-                auto place = [&](const auto &v) {
-                    const size_t o = buf.size(), bytes = sizeof(v[0]) * v.size();
-                    buf.resize(o + (bytes + sizeof(int4) - 1) / sizeof(int4), make_int4(0, 0, 0, 0));
-                    if (bytes) std::memcpy(buf.data() + o, v.data(), bytes);
-                    return o;
-                };
-                const size_t o_info = place(rinfo), o_val = place(gval), o_off = place(goff), o_width = place(gwidth),
-                             o_row = place(grow), o_col = place(gcol);
-                const int4 *base = nullptr;
-                up_(buf, &base);
-                if (st == MQCT_OK) {
-                    D.row_info = base + o_info;
-                    D.g_val = reinterpret_cast<const float2 *>(base + o_val);
-                    D.g_off = reinterpret_cast<const int *>(base + o_off);
-                    D.g_width = reinterpret_cast<const int *>(base + o_width);
-                    D.grp_row = reinterpret_cast<const int *>(base + o_row);
-                    D.g_col = reinterpret_cast<const unsigned short *>(base + o_col);
-                }
+                up_(grow, &D.grp_row);
+                up_(goff, &D.g_off);
+                up_(gwidth, &D.g_width);
+                up_(gval, &D.g_val);
+                up_(gcol, &D.g_col);
+                up_(rinfo, &D.row_info);
             }
             up_(aupf, &D.aupf);
             up_(adnf, &D.adnf);
