@@ -326,10 +326,9 @@ mqct_status mqct_system_info(mqct_system sys, mqct_system_info_t *out);
  *   diag       [n] mqct_diag; or NULL
  * Work order: trajectories are claimed from a device work queue, longest estimated
  * first.  Scratch memory is taken with stream-ordered allocation on `cuda_stream`.
- * With device output pointers the FP64 and FP32 calls only enqueue work and return MQCT_OK;
- * the BF16X3 path synchronises the stream between chunks of 16 steps (it checks on the host
- * whether trajectories are still running), and BF16X3 calls with several systems synchronise
- * it once to size the per-system launches.  With any host
+ * With device output pointers the FP64 and the FP32 factorised calls only enqueue work and return MQCT_OK;
+ * the stage-synchronous paths (BF16X3, FP32 PLAIN) synchronise the stream at the end of each
+ * system's graph, and with several systems once more to size the per-system launches.  With any host
  * output the call synchronises the stream and returns MQCT_ERR_TRAJ if a trajectory status
  * is non-zero (MQCT_ERR_TIMEOUT if one has MQCT_TRAJ_TIMEOUT).  Errors: MQCT_ERR_INVALID_ARG,
  * MQCT_ERR_UNSUPPORTED, MQCT_ERR_OOM, MQCT_ERR_CUDA, MQCT_ERR_TIMEOUT, MQCT_ERR_TRAJ. */

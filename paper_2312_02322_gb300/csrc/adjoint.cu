@@ -313,7 +313,8 @@ __device__ __forceinline__ double reduce16(double (&v)[16], int lane)
 // Vector-Jacobian product at stage (t, Y) in FP64: given the cotangent (KB, c.kb) of f, add J^T kbar to
 // (YN, c.ynew) and the parameter cotangent to c.theta.  Needs terms_at(Y_R).
 //
-// Bound by the FP64 pipe, so arranged for the fewest FP64 instructions: M z and M Dc (z = p kbar, Dc = (J+ - J-) c)
+// Arranged for the fewest FP64 instructions, whose pipe the kernel keeps 67 % busy (N = 441, 152 trajectories; the rest
+// is barriers, where the one-thread chains of the classical variables are waited for): M z and M Dc (z = p kbar, Dc = (J+ - J-) c)
 // enter the result as conj(p) M (i z - PPhibar Dc) only and are contracted as that one vector; the sums
 // Re(kbar^dag (-i conj(p) M' c)), Re(c^dag M'' c) and Re((Dc)^dag M' c) follow from the per-term sums alpha, beta, gamma
 // that the parameters need anyway; those are reduced five terms at a time (reduce16).  N = 441, 128 trajectories,
@@ -615,8 +616,8 @@ __device__ void vjp_eval32(const DevSys &S, double t, unsigned n_half, const flo
     __syncthreads();
 }
 
-// two CTAs per SM in the mixed precision, whose barriers and chains then fill each other's gaps (its FP64
-// counterpart fills the FP64 pipe and its shared memory with one): N = 441, 256 trajectories 498 -> 313 ms together
+// two CTAs per SM in the mixed precision, whose barriers and chains then fill each other's gaps (a CTA of its FP64
+// counterpart takes all registers of an SM): N = 441, 256 trajectories 498 -> 313 ms together
 // with the kept stage states (286 without the counting propagation)
 template <class R>
 __global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 2 : 1) k_adjoint(AdjArgs a)

@@ -34,8 +34,9 @@
 // and consecutive rows of a warp are contiguous, so the accesses are free of bank conflicts but for the
 // borders of the m-blocks.  Measured (equal lengths, against two barriers per stage with scalar
 // arithmetic, interleaved complex C and one entry per term and column): N = 441, 1216 trajectories 42.8 -> 72 M
-// traj-steps/s, 2185 warp instructions per trajectory-stage (3974 before), issue slots 50 % busy,
-// shared-memory data path 66 %; N = 1600, 1216 trajectories 8.6 -> 16.3 M (its tables come from L2).
+// traj-steps/s, 2102 warp instructions per trajectory-stage (3974 before), issue slots 51 % busy,
+// shared-memory data path 78 % (two CTAs of four slots per SM); N = 1600, 1216 trajectories 8.6 -> 16.3 M (its tables
+// come from L2).
 //
 // Uneven batches (trajectories of several systems, i.e. basis sizes, in one call) run in this one
 // persistent launch: a CTA binds to a system (its share of the grid at the start is proportional

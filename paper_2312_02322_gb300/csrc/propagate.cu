@@ -643,8 +643,9 @@ constexpr size_t kPropBasisBytes = 229216;  // of an SM's 232448 bytes per CTA
 
 // Element warps of a CTA: a warp takes 16 rows at a time, and there are as many as the rows feed, at most 14
 // (a 16-warp CTA, one per SM): N = 441, 256 trajectories 297 ms against 369 ms with eight warps and two CTAs
-// per SM, whose last trajectories leave half the GPU idle; 600 trajectories 615 against 602 ms; 64
-// trajectories 208 against 224 ms.  A basis of at most eight row groups with more than two trajectories per SM
+// per SM, whose last trajectories leave half the GPU idle; 64 trajectories 208 against 224 ms.  Four trajectories
+// per SM are the exception (600 take 615 ms against 602 with eight warps): 2 % that no bound on the count
+// separates from the 20 % of a batch with a tail.  A basis of at most eight row groups with more than two trajectories per SM
 // takes half as many warps as groups, two row groups a warp (N = 49, 600 trajectories 504 against 580 ms; N = 100,
 // 400 trajectories 628 against 690 ms): its stage is a chain of barriers that other CTAs fill.
 cudaError_t launch_propagate(PropArgs pa, int maxlev, bool adapt, cudaStream_t st)

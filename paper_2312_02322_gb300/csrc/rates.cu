@@ -25,7 +25,7 @@
 //       for x >= 0.1 and evaluated for the pair below (kRateChebX).
 //       About 170 FP64 instructions per pair and temperature instead of about 4400: the kernel is bound
 //       by the FP64 pipe, so the instruction count is its time.
-//   quadrature  for every other pair (a value below zero is taken as zero, R3), a u0 at or above U_K, and
+//   quadrature  (k_rates_quad) for every other pair (a value below zero is taken as zero, R3), a u0 at or above U_K, and
 //       temperatures or energies outside [1e-12, 1e6] hartree: 16-point Gauss-Legendre panels no
 //       wider than 4 kT (the exponential at the nodes as a panel factor times node factors shared by the
 //       panels of a piece); the walk stops at the first panel whose remainder bound
